@@ -4,41 +4,26 @@
 //
 //   out = s * A_y . in . A_x^T,   A[u][j] = exp(-+ 2 pi i X_j U_u)
 //
-// evaluated as two batched complex GEMMs. The bases are generated on the device in FP64
-// (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64 constant, reduced
-// to its fractional cycle before sincospi) and rounded to complex64.
+// evaluated as two batched GEMMs: on the CUDA cores over even / odd halves with real bases
+// (fold.cuh), on the tensor cores over split complex operands. The bases are generated on the
+// device in FP64 (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64
+// constant, reduced to its fractional cycle before sincospi) and rounded.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 #include <vector>
 
 #include "capi_common.h"
 #include "fft_engine.cuh"
-#include "mft_gemm.cuh"
+#include "fold.cuh"
 #include "tc_gemm.cuh"
 #include "tcx_gemm.cuh"
 
 using namespace coro;
 
 namespace {
-
-// basis[b][u][j] = exp(sign 2 pi i (j - n/2)(u - m/2) c_b), c_b = du_b / npix.
-template <typename C>
-__global__ void mft_basis_kernel(C* basis, int m, int n, const double* __restrict__ c, int sign) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int u = blockIdx.y;
-    const int b = blockIdx.z;
-    if (j >= n) return;
-    const long long jj = (long long)j - n / 2, uu = (long long)u - m / 2;
-    double cyc = (double)(jj * uu) * c[b];
-    cyc -= rint(cyc);
-    double s, co;
-    sincospi(2.0 * cyc, &s, &co);
-    if (sign < 0) s = -s;
-    using R = typename real_of<C>::type;
-    basis[((size_t)b * m + u) * n + j] = mk<C>((R)co, (R)s);
-}
 
 coro_status check_mft_wf(const char* fn, const coro_wavefront* wf) {
     if (!wf || !wf->data) { coro::set_error("%s: wavefront or data is NULL", fn); return CORO_EINVAL; }
@@ -179,68 +164,46 @@ coro_status mft_ext(coro_ctx ctx, const coro_wavefront* in, int direction, int m
     return CORO_OK;
 }
 
-// CUDA-core MFT: complex64 with FP32 arithmetic or complex128 with FP64 arithmetic.
+// CUDA-core MFT: complex64 with FP32 arithmetic or complex128 with FP64 arithmetic, on even / odd
+// halves (fold.cuh): fold and bases in one launch, two contractions, the expansion.
 template <typename C>
 coro_status mft_cuda_cores(coro_ctx ctx, const coro_wavefront* in, int direction, int m, const std::vector<double>& c,
                            coro_wavefront* out) {
-    using Real = typename real_of<C>::type;
-    using Desc = typename std::conditional<std::is_same<C, float2>::value, GemmDesc, ZGemmDesc>::type;
+    using R = typename real_of<C>::type;
     coro_status st = CORO_OK;
-    const int batch = in->batch;
-    auto gemm = [&](const Desc& g) -> cudaError_t {
-        if constexpr (std::is_same<C, float2>::value) return launch_cgemm(g, batch, CORO_MFT_FP32, ctx->stream);
-        else return launch_zgemm(g, batch, ctx->stream);
-    };
-    // focal-plane side has m (forward) or in->n (inverse) samples; pupil side the other
-    const int nf = direction < 0 ? m : in->n;     // focal samples per axis
-    const int np = direction < 0 ? in->n : m;     // pupil samples per axis
-    const size_t basis_elems = (size_t)batch * nf * np;
-    const size_t t_elems = (size_t)batch * (direction < 0 ? (size_t)np * nf : (size_t)nf * np);
-    C* work = (C*)coro::ctx_work(ctx, (basis_elems + t_elems) * sizeof(C), &st);
+    const int batch = in->batch, n = in->n, hn = fold_len(n), hm = fold_len(m), ldw = fold_ldw(hm);
+    // items per round: the contractions carry item x parity (x K split) in grid z
+    const int round = batch < 4096 ? batch : 4096;
+    auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    const size_t f_bytes = align((size_t)round * 4 * hn * hn * sizeof(C)), w_bytes = align((size_t)round * 2 * hn * ldw * sizeof(R));
+    const size_t y_bytes = align((size_t)round * 4 * hn * hm * sizeof(C)), t_bytes = align((size_t)round * 4 * hm * hm * sizeof(C));
+    size_t part_elems = 0;
+    if (std::is_same<C, float2>::value)
+        part_elems = std::max(fold_part_elems(2 * hn, hm, hn, round), fold_part_elems(2 * hm, hm, hn, round));
+    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, f_bytes + w_bytes + y_bytes + t_bytes + part_elems * sizeof(C), &st);
     if (!work) return st;
-    C* basis = work;
-    C* tmp = work + basis_elems;
-    void* c_d = coro::upload_async(ctx, c.data(), c.size() * sizeof(double), &st);
-    if (!c_d) return st;
-    dim3 bg((np + 127) / 128, nf, batch);
-    mft_basis_kernel<C><<<bg, 128, 0, ctx->stream>>>(basis, nf, np, (const double*)c_d, direction < 0 ? -1 : 1);
-    cudaError_t e = cudaGetLastError();
-    coro::free_async(ctx, c_d);
-    if (e != cudaSuccess) return coro::cuda_fail(e, "mft_basis_kernel");
-
-    const C* x = (const C*)in->data;
-    C* y = (C*)out->data;
-    const long long sb = (long long)nf * np;   // basis batch stride
-    Desc g1{}, g2{};
-    if (direction < 0) {
-        // T[i][u] = sum_j in[i][j] A[u][j]            (M = np, N = nf, K = np)
-        g1 = Desc{np, nf, np, x, (long long)np * np, np, false, basis, sb, np, true,
-                      tmp, (long long)np * nf, nf, (Real)1};
-        // out[v][u] = s sum_i A[v][i] T[i][u]         (M = nf, N = nf, K = np)
-        g2 = Desc{nf, nf, np, basis, sb, np, false, tmp, (long long)np * nf, nf, false,
-                      y, (long long)nf * nf, nf, (Real)0};
-    } else {
-        // T[v][j] = sum_u in[v][u] B[u][j]            (M = nf, N = np, K = nf)
-        g1 = Desc{nf, np, nf, x, (long long)nf * nf, nf, false, basis, sb, np, false,
-                      tmp, (long long)nf * np, np, (Real)1};
-        // out[i][j] = s sum_v B[v][i] T[v][j]         (M = np, N = np, K = nf)
-        g2 = Desc{np, np, nf, basis, sb, np, true, tmp, (long long)nf * np, np, false,
-                      y, (long long)np * np, np, (Real)0};
+    C* F = (C*)work;
+    R* W = (R*)(work + f_bytes);
+    C* Y = (C*)(work + f_bytes + w_bytes);
+    C* T = (C*)(work + f_bytes + w_bytes + y_bytes);
+    C* part = part_elems ? (C*)(work + f_bytes + w_bytes + y_bytes + t_bytes) : nullptr;
+    cudaError_t e = cudaSuccess;
+    for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += round) {
+        const int nb = std::min(round, batch - b0);
+        e = fold_prepare<C>((const C*)in->data + (size_t)b0 * n * n, n, hn, -1, F, c.data() + b0, hn, hm, W, nb, ctx->stream);
+        FoldGemm<C> g{2 * hn, hm, hn, nb, F, (long long)4 * hn * hn, W, (long long)2 * hn * ldw, ldw, Y, (long long)4 * hn * hm,
+                      FOLD_PLAIN, 0, (R)1, nullptr, 0};
+        if (e == cudaSuccess) e = fold_gemm(g, part, ctx->stream);
+        g.M = 2 * hm;
+        g.X = Y;
+        g.sX = (long long)4 * hn * hm;
+        g.Y = T;
+        g.sY = (long long)4 * hm * hm;
+        if (e == cudaSuccess) e = fold_gemm(g, part, ctx->stream);
+        if (e == cudaSuccess)
+            e = fold_expand<C>(T, m, direction < 0 ? -1 : 1, c.data() + b0, (C*)out->data + (size_t)b0 * m * m, nb, ctx->stream);
     }
-    std::vector<Real> scale(batch);
-    for (int b = 0; b < batch; ++b) scale[b] = (Real)c[b];
-    void* s_d = coro::upload_async(ctx, scale.data(), batch * sizeof(Real), &st);
-    if (!s_d) return st;
-    g2.scale_per_item = (const Real*)s_d;
-    e = gemm(g1);
-    if (e == cudaSuccess) e = gemm(g2);
-    coro::free_async(ctx, s_d);
-    if (e == cudaErrorNotSupported) {
-        coro::set_error("coro_propagate_mft: CUDA-core GEMM not available in this build");
-        return CORO_ENOTIMPL;
-    }
-    if (e != cudaSuccess) return coro::cuda_fail(e, "mft gemm");
-    return CORO_OK;
+    return e == cudaSuccess ? CORO_OK : coro::cuda_fail(e, "mft (folded)");
 }
 
 }  // namespace
