@@ -8,11 +8,19 @@
 //   G4  E_D = Lyot . (E_A - s_occ (Z3 . B^T)^T)       Babinet, in place over E_A's planes
 //   G5  Z5 = (E_D . A_det^T)^T
 //   G6  I = |s_det (Z5 . A_det^T)^T|^2 / peak,   S = sum over the dark-hole annulus of I
-// Every G is one launch of the split-precision tensor-core GEMM (tc_gemm.cu) over the whole
-// batch; the spot, the Babinet subtraction, the Lyot stop, the intensity and the dark-hole sum
-// are epilogues, so the only extra pass is the split of E_A.
+// Every G is one launch of a split-precision tensor-core GEMM over the whole batch; the spot, the
+// Babinet subtraction and the Lyot stop are epilogues.
+//
+// The chain runs on even / odd halves with real bases (Folded below; ft_gemm.cuh): the field is
+// folded once into its four parity classes, every plane is kept only as far as its mask reaches
+// (E_B inside the spot, E_D inside the stop), and the classes meet again at the detector. For the
+// 1024^2 / 256^2 / 512^2 system that is 0.99 G real multiply-adds per image and product term
+// instead of 4.4 G (the complex GEMMs over the known supports). Plans whose masks reach the
+// unpaired edge sample of an even array (a stop as wide as the pupil array, a spot or a dark hole
+// as wide as its plane) mix the classes there and keep the complex GEMMs (tc_gemm.cu, tcx_gemm.cu).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <map>
@@ -20,6 +28,8 @@
 #include <vector>
 
 #include "capi_common.h"
+#include "fold.cuh"
+#include "ft_gemm.cuh"
 #include "tc_gemm.cuh"
 #include "tcx_gemm.cuh"
 
@@ -32,7 +42,25 @@ struct Buf {
     size_t bytes = 0;
 };
 
+// The folded chain's operands, bases, contractions and item tables. Extents (samples from the axis
+// on): h pupil, s spot (per item; sm the largest), l Lyot stop, d detector, dd dark hole (dm).
+enum FoldStage { F_G1, F_G2, F_G3, F_G4, F_G5, F_G6, F_DET, F_G5G, F_SEED, F_H1, F_H2, F_G1G, F_G2G, F_G3G, F_G4G, F_STAGES };
+
+struct Folded {
+    int fmt = FT_TF32, h = 0, sm = 0, l = 0, d = 0, dm = 0, stop = 0;
+    FtOperand FA, Y1, ZB, Y3, D, Y5, W1, W2, W3;
+    FtOperand XS, Z4, W4, Y1g, Y3g;    // adjoint
+    void* T = nullptr;                 // classes at the detector, FP32 (FT_EXT: two-float)
+    float* GA = nullptr;               // classes of the pupil gradient
+    FtGemm g[F_STAGES];
+    std::vector<FtItem> host;          // [F_STAGES][batch]
+    FtItem* dev = nullptr;
+    double* dh_part = nullptr;         // dark-hole partial sums and their counters
+    unsigned* dh_count = nullptr;
+};
+
 struct LyotPlan : coro_plan_s {
+    std::unique_ptr<Folded> f;
     coro_ctx ctx = nullptr;
     bool bf16 = false;
     bool ext = false;                  // CORO_MFT_EXT: sliced BF16 operands (tcx_gemm.cu)
@@ -59,7 +87,7 @@ struct LyotPlan : coro_plan_s {
     double* peak64 = nullptr;          // [batch] (CORO_MFT_EXT)
     int device = 0;                    // kept so that destruction never touches the context
     int kind() const override { return 2; }
-    int launches() const override { return 7; }
+    int launches() const override { return f ? 8 : 7; }
     int timing_units() const override { return 6; }     // the stages of execute_range
     ~LyotPlan() override {
         DeviceGuard g(device);
@@ -115,6 +143,200 @@ int clamp_thr(long long v) { return v > 0x3fffffffLL ? 0x3fffffff : (int)v; }
 
 coro_status tune_tile(LyotPlan* p);
 
+// Samples from the axis on that a disk of k2 <= thr reaches on an n-sample axis.
+int disk_extent(long long thr, int n) { return (int)std::min<long long>(isqrt_floor(thr) + 1, fold_len(n)); }
+// Whether a disk leaves the unpaired sample of an even axis (index -n/2) out.
+bool disk_paired(long long thr, int n) { return n % 2 || thr < (long long)(n / 2) * (n / 2); }
+
+// The folded chain serves every plan whose three masks leave the unpaired samples out.
+bool foldable(const coro_lyot_desc* d) {
+    if (!disk_paired(disk_threshold(0.5 * d->lyot_frac, 1.0 / d->npix, false), d->n)) return false;
+    for (int b = 0; b < d->batch; ++b) {
+        const coro_lyot_item& it = d->items[b];
+        if (!disk_paired(disk_threshold(it.spot_radius, it.du_occ, false), it.m_occ)) return false;
+        if (!disk_paired(disk_threshold(it.dh_out, it.du_det, false), d->m_det)) return false;
+    }
+    return true;
+}
+
+// Float planes [item][2][2][2][R][R] of extent `ext` as a destination (whole sectors, as operands).
+FtOperand float_planes(void* base, int ext) {
+    FtOperand o;
+    o.base = base;
+    o.R = o.ld = ft_pitch(FT_TF32, ext);
+    o.stride = (long long)8 * o.R * o.ld;
+    return o;
+}
+
+bool alloc_operand(LyotPlan* p, FtOperand& o, coro_status* st) {
+    o.base = p->alloc(ft_bytes(p->f->fmt, o), st);
+    return o.base != nullptr;
+}
+
+// The contractions' maps and tiles (again after a change of the tile width).
+cudaError_t make_gemms(LyotPlan* p) {
+    Folded& f = *p->f;
+    const int B = p->batch, nt = p->ext ? 2 * p->tile_n : 128;
+    cudaError_t e = cudaSuccess;
+    auto make = [&](int st, const FtOperand& x, const FtOperand& w, int max_n) {
+        if (e == cudaSuccess) e = ft_make(f.fmt, x, w, B, max_n, nt, &f.g[st]);
+    };
+    make(F_G1, f.FA, f.W1, f.sm);
+    make(F_G2, f.Y1, f.W1, f.sm);
+    make(F_G3, f.ZB, f.W2, f.l);
+    make(F_G4, f.Y3, f.W2, f.l);
+    make(F_G5, f.D, f.W3, f.d);
+    make(F_G6, f.Y5, f.W3, f.d);
+    if (p->grad_ready) {
+        make(F_G5G, f.D, f.W3, f.dm);
+        make(F_SEED, f.Y5, f.W3, f.dm);
+        make(F_H1, f.XS, f.W4, f.l);
+        make(F_H2, f.Z4, f.W4, f.l);
+        make(F_G1G, f.D, f.W1, f.sm);
+        make(F_G2G, f.Y1g, f.W1, f.sm);
+        make(F_G3G, f.ZB, f.W2, f.h);
+        make(F_G4G, f.Y3g, f.W2, f.h);
+    }
+    return e;
+}
+
+coro_status make_folded(LyotPlan* p, const coro_lyot_desc* d) {
+    p->f.reset(new Folded);
+    Folded& f = *p->f;
+    const int B = d->batch, n = d->n, all = 0x7fffffff;
+    f.fmt = p->ext ? FT_EXT : p->bf16 ? FT_BF16 : FT_TF32;
+    f.h = fold_len(n);
+    f.d = fold_len(d->m_det);
+    f.stop = clamp_thr(disk_threshold(0.5 * d->lyot_frac, 1.0 / d->npix, false));
+    f.l = disk_extent(f.stop, n);
+    p->pupil_ld = n;
+    p->pupil_bstride = (long long)n * n;
+    f.host.resize((size_t)F_STAGES * B);
+    // one basis per distinct sampling: occulter (extent, pitch) and detector pitch
+    std::map<std::pair<int, double>, int> occ;
+    std::map<double, int> det;
+    for (int b = 0; b < B; ++b) {
+        const coro_lyot_item& it = d->items[b];
+        const int spot = clamp_thr(disk_threshold(it.spot_radius, it.du_occ, false)), s = disk_extent(spot, it.m_occ);
+        const int dh_lo = clamp_thr(disk_threshold(it.dh_in, it.du_det, true) + 1);
+        const int dh_hi = clamp_thr(disk_threshold(it.dh_out, it.du_det, false)), dd = disk_extent(dh_hi, d->m_det);
+        const double so = it.du_occ / d->npix, sd = it.du_det / d->npix;
+        const int oi = occ.emplace(std::make_pair(s, it.du_occ), (int)occ.size()).first->second;
+        const int di = det.emplace(it.du_det, (int)det.size()).first->second;
+        f.sm = std::max(f.sm, s);
+        f.dm = std::max(f.dm, dd);
+        auto put = [&](int st, int K, int N, int H, int w, int thr_in, int thr_out, double scale) {
+            f.host[(size_t)st * B + b] = FtItem{K, N, H, w, thr_in, thr_out, dh_lo, scale, 1.0};
+        };
+        put(F_G1, f.h, s, f.h, oi, -1, all, 1.0);
+        put(F_G2, f.h, s, s, oi, -1, spot, 1.0);
+        put(F_G3, s, f.l, s, oi, spot, all, 1.0);
+        put(F_G4, s, f.l, f.l, oi, -1, f.stop, so * so);
+        put(F_G5, f.l, f.d, f.l, di, f.stop, all, 1.0);
+        put(F_G6, f.l, f.d, f.d, di, -1, all, 1.0);
+        put(F_DET, 0, 0, 0, di, -1, dh_hi, sd);
+        // adjoint: the seed only inside the dark hole, back through the detector transform to the
+        // stop, then Babinet's block to the whole pupil
+        put(F_G5G, f.l, dd, f.l, di, f.stop, all, 1.0);
+        put(F_SEED, f.l, dd, dd, di, -1, dh_hi, sd);
+        put(F_H1, dd, f.l, dd, di, dh_hi, all, 1.0);
+        put(F_H2, dd, f.l, f.l, di, -1, f.stop, sd);
+        put(F_G1G, f.l, s, f.l, oi, f.stop, all, 1.0);
+        put(F_G2G, f.l, s, s, oi, -1, spot, 1.0);
+        put(F_G3G, s, f.h, s, oi, spot, all, 1.0);
+        put(F_G4G, s, f.h, f.h, oi, -1, all, so * so);
+    }
+    const int no = (int)occ.size(), nd = (int)det.size();
+    f.FA = ft_operand(f.fmt, B, f.h, f.h);
+    f.Y1 = ft_operand(f.fmt, B, f.sm, f.h);
+    f.ZB = ft_operand(f.fmt, B, f.sm, f.sm);
+    f.Y3 = ft_operand(f.fmt, B, f.l, f.sm);
+    f.D = ft_operand(f.fmt, B, f.l, f.l);
+    f.Y5 = ft_operand(f.fmt, B, f.d, f.l);
+    f.W1 = ft_basis_operand(f.fmt, no, f.sm, f.h);
+    f.W2 = ft_basis_operand(f.fmt, no, f.h, f.sm);
+    f.W3 = ft_basis_operand(f.fmt, nd, f.d, f.l);
+    coro_status st = CORO_OK;
+    for (FtOperand* o : {&f.FA, &f.Y1, &f.ZB, &f.Y3, &f.D, &f.Y5, &f.W1, &f.W2, &f.W3})
+        if (!alloc_operand(p, *o, &st)) return st;
+    f.T = p->alloc((size_t)B * float_planes(nullptr, f.d).stride * (p->ext ? sizeof(float2) : sizeof(float)), &st);
+    f.dev = f.T ? (FtItem*)p->alloc(f.host.size() * sizeof(FtItem), &st) : nullptr;
+    p->dh = f.dev ? (double*)p->alloc(B * sizeof(double), &st) : nullptr;
+    p->peak = p->dh ? (float*)p->alloc(B * sizeof(float), &st) : nullptr;
+    p->peak64 = p->peak ? (double*)p->alloc(B * sizeof(double), &st) : nullptr;
+    if (p->peak64) f.dh_part = (double*)p->alloc(B * ft_plane_parts(d->m_det) * sizeof(double), &st);
+    if (f.dh_part) f.dh_count = (unsigned*)p->alloc(B * sizeof(unsigned), &st);
+    if (!f.dh_count) return st;
+    cudaError_t e = cudaSuccess;
+    for (auto& kv : occ) {
+        const double c = kv.first.second / d->npix;
+        if (e == cudaSuccess) e = ft_basis(f.fmt, c, f.h, kv.first.first, f.W1, kv.second, p->ctx->stream);
+        if (e == cudaSuccess) e = ft_basis(f.fmt, c, kv.first.first, f.h, f.W2, kv.second, p->ctx->stream);
+    }
+    for (auto& kv : det) {
+        if (e == cudaSuccess) e = ft_basis(f.fmt, kv.first / d->npix, f.l, f.d, f.W3, kv.second, p->ctx->stream);
+        p->det_bases.push_back({kv.first, kv.second});
+    }
+    if (e == cudaSuccess) e = make_gemms(p);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(f.dev, f.host.data(), f.host.size() * sizeof(FtItem), cudaMemcpyHostToDevice, p->ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p->ctx->stream);
+    return e == cudaSuccess ? CORO_OK : cuda_fail(e, "coro_lyot_plan_create (folded)");
+}
+
+// One contraction of the folded chain into operand or float planes.
+cudaError_t fold_step(LyotPlan* p, int stage, int epi, const FtOperand& x, const FtOperand& dst, int weights = 0) {
+    const Folded& f = *p->f;
+    FtArgs a{};
+    a.items = f.dev + (size_t)stage * p->batch;
+    a.err = p->ctx->err;
+    a.R = x.R;
+    a.weights = weights;
+    a.dst = dst.base;
+    a.dst_bstride = dst.stride;
+    a.dst_R = dst.R;
+    a.dst_ld = dst.ld;
+    if (epi == FT_BABINET || epi == FT_DIFF) {
+        const FtOperand& b = epi == FT_BABINET ? f.FA : f.D;
+        a.base = b.base;
+        a.base_bstride = b.stride;
+        a.base_R = b.R;
+        a.base_ld = b.ld;
+        a.base_H = epi == FT_BABINET ? f.h : f.l;
+    }
+    a.dh_acc = p->dh;
+    return ft_launch(f.g[stage], epi, a, p->ctx->stream);
+}
+
+// Detector transform of the classes in D, and the plane.
+cudaError_t folded_detector(LyotPlan* p, float* intensity, void* field, bool track_peak) {
+    const Folded& f = *p->f;
+    cudaStream_t s = p->ctx->stream;
+    cudaError_t e = fold_step(p, F_G5, FT_SPLIT, f.D, f.Y5);
+    if (e == cudaSuccess) e = fold_step(p, F_G6, FT_FLOAT, f.Y5, float_planes(f.T, f.d));
+    if (e == cudaSuccess && track_peak) e = cudaMemsetAsync(p->peak, 0, p->batch * sizeof(float), s);
+    if (e == cudaSuccess && track_peak) e = cudaMemsetAsync(p->peak64, 0, p->batch * sizeof(double), s);
+    if (e != cudaSuccess) return e;
+    FtPlane pl{};
+    pl.items = f.dev + (size_t)F_DET * p->batch;
+    pl.T = f.T;
+    pl.ext = p->ext;
+    const FtOperand t = float_planes(f.T, f.d);
+    pl.R = t.R;
+    pl.ld = t.ld;
+    pl.bstride = t.stride;
+    pl.m = p->m_det;
+    pl.sign = -1;
+    pl.image = intensity;
+    pl.field = (float2*)field;
+    pl.dh = p->dh;
+    pl.dh_part = f.dh_part;
+    pl.dh_count = f.dh_count;
+    pl.peak = track_peak ? p->peak : nullptr;
+    pl.peak64 = track_peak ? p->peak64 : nullptr;
+    return ft_plane(pl, p->batch, s);
+}
+
 }  // namespace
 
 extern "C" coro_status coro_lyot_plan_create(coro_ctx ctx, const coro_lyot_desc* d, coro_plan* out) {
@@ -157,6 +379,16 @@ extern "C" coro_status coro_lyot_plan_create(coro_ctx ctx, const coro_lyot_desc*
     p->m_occ_max = m_occ_max;
     p->items.assign(d->items, d->items + d->batch);
     const int B = d->batch, n = d->n, md = d->m_det;
+    if (foldable(d)) {
+        const coro_status fs = make_folded(p.get(), d);
+        if (fs != CORO_OK) return fs;
+        if (p->ext && !(std::getenv("CORO_AUTOTUNE") && std::getenv("CORO_AUTOTUNE")[0] == '0')) {
+            const coro_status ts = tune_tile(p.get());
+            if (ts != CORO_OK) return ts;
+        }
+        *out = p.release();
+        return CORO_OK;
+    }
 
     // distinct bases: occulter (m_occ, du_occ) and detector du_det
     std::map<std::pair<int, double>, int> occ_id;
@@ -263,6 +495,15 @@ namespace {
 cudaError_t upload_det_items(LyotPlan* p, const double* peak_host) {
     const int B = p->batch;
     cudaStream_t s = p->ctx->stream;
+    if (p->f) {                                          // the detector plane's items and the seed's
+        cudaError_t e = cudaSuccess;
+        for (int st : {(int)F_DET, (int)F_SEED}) {
+            FtItem* h = p->f->host.data() + (size_t)st * B;
+            for (int b = 0; b < B; ++b) h[b].inv_peak = peak_host ? 1.0 / peak_host[b] : 1.0;
+            if (e == cudaSuccess) e = cudaMemcpyAsync(p->f->dev + (size_t)st * B, h, B * sizeof(FtItem), cudaMemcpyHostToDevice, s);
+        }
+        return e;
+    }
     if (peak_host) {
         std::vector<TcItem> g6(p->host_items.begin() + 5 * B, p->host_items.begin() + 6 * B);
         for (int b = 0; b < B; ++b) {
@@ -325,6 +566,23 @@ cudaError_t run_stages(LyotPlan* p, const void* pupil, float* intensity, void* f
         if (ev && e == cudaSuccess) e = record_timing_event(ev[i], s);
     };
     mark(0);
+    if (p->f) {
+        const Folded& f = *p->f;
+        auto step = [&](int at, int stage, int epi, const FtOperand& x, const FtOperand& dst, int weights) {
+            if (e == cudaSuccess && at >= first && at <= last) e = fold_step(p, stage, epi, x, dst, weights);
+            mark(at + 1);
+        };
+        if (first <= 0 && last >= 0)
+            e = ft_fold(f.fmt, (const float2*)pupil, p->pupil_bstride, p->pupil_ld, n, f.h, -1, f.FA, s);
+        mark(1);
+        step(1, F_G1, FT_SPLIT, f.FA, f.Y1, 0);
+        step(2, F_G2, FT_SPLIT, f.Y1, f.ZB, 1);          // x spot
+        step(3, F_G3, FT_SPLIT, f.ZB, f.Y3, 0);
+        step(4, F_G4, FT_BABINET, f.Y3, f.D, 1);         // Babinet, x Lyot
+        if (e == cudaSuccess && first <= 5 && last >= 5) e = folded_detector(p, intensity, field, false);
+        mark(6);
+        return e;
+    }
     auto gemm = [&](int gi, int epi, const CUtensorMap& mx, const CUtensorMap& mw, const TcOperand& dst, int mm, int nn, int kk) {
         if (e != cudaSuccess || gi + 1 < first || gi + 1 > last) return;
         TcArgs a{};
@@ -359,6 +617,7 @@ namespace {
 
 // Re-encode the basis maps for the plan's tile width (their boxes have tile_n rows).
 cudaError_t remap_bases(LyotPlan* p) {
+    if (p->f) return make_gemms(p);
     cudaError_t e = p->map(p->W1, true, &p->mW1);
     if (e == cudaSuccess) e = p->map(p->W2, true, &p->mW2);
     if (e == cudaSuccess) e = p->map(p->W3, true, &p->mW3);
@@ -528,7 +787,13 @@ extern "C" coro_status coro_lyot_plan_flops(coro_plan plan, double* useful, doub
     const int epi[6] = {TC_EPI_SPLITT, TC_EPI_SPLITT, TC_EPI_SPLITT, TC_EPI_BABINET, TC_EPI_SPLITT, TC_EPI_INTENSITY};
     const int mm[6] = {n, mo, mo, n, n, md}, nn[6] = {mo, mo, n, n, md, md};
     double u = 0, is = 0;
-    for (int g = 0; g < 6; ++g) {
+    if (p->f) {
+        const Folded& f = *p->f;
+        const int fe[6] = {FT_SPLIT, FT_SPLIT, FT_SPLIT, FT_BABINET, FT_SPLIT, FT_FLOAT};
+        const FtOperand* x[6] = {&f.FA, &f.Y1, &f.ZB, &f.Y3, &f.D, &f.Y5};
+        for (int g = 0; g < 6; ++g) ft_count_flops(f.g[g], fe[g], f.host.data() + (size_t)g * B, x[g]->R, &u, &is);
+    }
+    for (int g = 0; g < 6 && !p->f; ++g) {
         if (p->ext) tcx_count_flops(epi[g], p->host_items.data() + (size_t)g * B, B, mm[g], nn[g], &u, &is, p->tile_n);
         else tc_count_flops(p->bf16, epi[g], p->host_items.data() + (size_t)g * B, B, mm[g], nn[g], &u, &is);
     }
@@ -546,9 +811,11 @@ extern "C" coro_status coro_lyot_plan_peak(coro_plan plan, const void* pupil, do
     DeviceGuard g(p->ctx->device);
     cudaStream_t s = p->ctx->stream;
     // occulter removed: E_D = E_A . Lyot stop, then the detector MFT
-    cudaError_t e = p->split((const float2*)pupil, p->pupil_bstride, p->pupil_ld, p->XA, p->keep_lyot);
+    cudaError_t e = p->f ? ft_fold(p->f->fmt, (const float2*)pupil, p->pupil_bstride, p->pupil_ld, n, p->f->l, p->f->stop,
+                                   p->f->D, s)
+                         : p->split((const float2*)pupil, p->pupil_bstride, p->pupil_ld, p->XA, p->keep_lyot);
     if (e == cudaSuccess) e = upload_det_items(p, nullptr);
-    if (e == cudaSuccess) e = detector_gemms(p, nullptr, nullptr, true);
+    if (e == cudaSuccess) e = p->f ? folded_detector(p, nullptr, nullptr, true) : detector_gemms(p, nullptr, nullptr, true);
     std::vector<float> pk(B);
     std::vector<double> pk64(B);
     if (e == cudaSuccess) e = cudaMemcpyAsync(pk.data(), p->peak, B * sizeof(float), cudaMemcpyDeviceToHost, s);
@@ -583,6 +850,25 @@ coro_status prepare_gradient(LyotPlan* p) {
     coro_status st = CORO_OK;
     const int B = p->batch, n = p->n, md = p->m_det;
     const int nd = (int)p->det_bases.size();
+    if (p->f) {
+        Folded& f = *p->f;
+        f.XS = ft_operand(f.fmt, B, f.dm, f.dm);
+        f.Z4 = ft_operand(f.fmt, B, f.l, f.dm);
+        f.W4 = ft_basis_operand(f.fmt, nd, f.l, f.dm);
+        f.Y1g = ft_operand(f.fmt, B, f.sm, f.l);
+        f.Y3g = ft_operand(f.fmt, B, f.h, f.sm);
+        for (FtOperand* o : {&f.XS, &f.Z4, &f.W4, &f.Y1g, &f.Y3g})
+            if (!alloc_operand(p, *o, &st)) return st;
+        f.GA = (float*)p->alloc((size_t)B * float_planes(nullptr, f.h).stride * sizeof(float), &st);
+        if (!f.GA) return st;
+        cudaError_t e = cudaSuccess;
+        for (auto& db : p->det_bases)
+            if (e == cudaSuccess) e = ft_basis(f.fmt, db.first / p->npix, f.dm, f.l, f.W4, db.second, p->ctx->stream);
+        p->grad_ready = true;
+        if (e == cudaSuccess) e = make_gemms(p);
+        if (e != cudaSuccess) { p->grad_ready = false; return cuda_fail(e, "coro_lyot_plan_gradient: set-up"); }
+        return CORO_OK;
+    }
     if (!p->make(p->XS, B, md, md, &st) || !p->make(p->Z4, B, n, md, &st) || !p->make(p->W4, nd, n, md, &st, true))
         return st;
     p->seed = (float2*)p->alloc((size_t)B * md * md * sizeof(float2), &st);
@@ -622,6 +908,28 @@ extern "C" coro_status coro_lyot_plan_gradient(coro_plan plan, const void* pupil
     // forward (stages 0-4), then the detector MFT writing the seed mask . E_det / peak
     cudaError_t e = run_stages(p, pupil, nullptr, nullptr, 0, 4);
     if (e == cudaSuccess) e = upload_det_items(p, peak);
+    if (p->f) {
+        // classes of the seed inside the dark hole, back to the stop, Babinet's block, the plane
+        const Folded& f = *p->f;
+        auto step = [&](int stage, int epi, const FtOperand& x, const FtOperand& dst, int weights) {
+            if (e == cudaSuccess) e = fold_step(p, stage, epi, x, dst, weights);
+        };
+        if (e == cudaSuccess) e = cudaMemsetAsync(p->dh, 0, B * sizeof(double), s);
+        step(F_G5G, FT_SPLIT, f.D, f.Y5, 0);
+        step(F_SEED, FT_SEED, f.Y5, f.XS, 1);
+        if (e == cudaSuccess && dh_out) e = cudaMemcpyAsync(dh_out, p->dh, B * sizeof(double), cudaMemcpyDeviceToHost, s);
+        step(F_H1, FT_SPLIT, f.XS, f.Z4, 0);
+        step(F_H2, FT_SPLIT, f.Z4, f.D, 1);              // x Lyot -> classes of G_C in D
+        step(F_G1G, FT_SPLIT, f.D, f.Y1g, 0);
+        step(F_G2G, FT_SPLIT, f.Y1g, f.ZB, 1);           // x spot
+        step(F_G3G, FT_SPLIT, f.ZB, f.Y3g, 0);
+        const FtOperand ga = float_planes(f.GA, f.h);
+        step(F_G4G, FT_DIFF, f.Y3g, ga, 1);
+        if (e == cudaSuccess)
+            e = ft_unfold(f.GA, ga.R, ga.ld, ga.stride, n, B, (float2*)grad, grad_ld, grad_bstride, s);
+        if (e == cudaSuccess && dh_out) e = cudaStreamSynchronize(s);
+        return e == cudaSuccess ? CORO_OK : cuda_fail(e, "coro_lyot_plan_gradient");
+    }
     if (e == cudaSuccess) e = detector_gemms(p, nullptr, nullptr, false, p->seed);
     if (e == cudaSuccess && dh_out) e = cudaMemcpyAsync(dh_out, p->dh, B * sizeof(double), cudaMemcpyDeviceToHost, s);
     // adjoint: G_D = IMFT_det(seed); G_C = Lyot . G_D; G_A = G_C - IMFT_occ(spot . MFT_occ(G_C))

@@ -4,9 +4,8 @@
 //
 //   out = s * A_y . in . A_x^T,   A[u][j] = exp(-+ 2 pi i X_j U_u)
 //
-// evaluated as two batched GEMMs: on the CUDA cores over even / odd halves with real bases
-// (fold.cuh), on the tensor cores over split complex operands. The bases are generated on the
-// device in FP64 (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64
+// evaluated as two batched GEMMs over even / odd halves with real bases: on the CUDA cores
+// (fold.cuh) or on the tensor cores (ft_gemm.cuh). The bases are generated on the device in FP64 (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64
 // constant, reduced to its fractional cycle before sincospi) and rounded.
 #include <cuda_runtime.h>
 
@@ -18,8 +17,7 @@
 #include "capi_common.h"
 #include "fft_engine.cuh"
 #include "fold.cuh"
-#include "tc_gemm.cuh"
-#include "tcx_gemm.cuh"
+#include "ft_gemm.cuh"
 
 using namespace coro;
 
@@ -33,134 +31,82 @@ coro_status check_mft_wf(const char* fn, const coro_wavefront* wf) {
     return CORO_OK;
 }
 
-// Split-precision tensor-core MFT: Y1 = X . W^T written transposed and split, then
-// out = s (Y1^T . W^T)^T, with W[r][k] = exp(-+2 pi i r' k' du/npix) the MFT basis.
+// Tensor-core MFT (3xTF32, 3xBF16, EXT) on even / odd halves (ft_gemm.cuh): fold, bases, two
+// contractions to the parity classes of the result, and the plane of all signs.
 coro_status mft_tensor_core(coro_ctx ctx, const coro_wavefront* in, int direction, int m, const std::vector<double>& c,
-                            bool bf16, coro_wavefront* out) {
+                            int fmt, coro_wavefront* out) {
     coro_status st = CORO_OK;
-    const int batch = in->batch;
-    const int nin = in->n;                       // X1 rows = cols
-    const int nout = m;                          // W rows, output size
-    const size_t es = tc_elem_size(bf16);
-    const int ld = tc_ld(nin, bf16);
-    const size_t x_bytes = (size_t)4 * batch * nin * ld * es;
-    const size_t w_bytes = (size_t)4 * batch * nout * ld * es;
-    const size_t z_bytes = w_bytes;
+    const int batch = in->batch, n = in->n, hn = fold_len(n), hm = fold_len(m);
+    FtOperand X = ft_operand(fmt, batch, hn, hn), W = ft_basis_operand(fmt, batch, hm, hn), Y = ft_operand(fmt, batch, hm, hn);
+    const int ld_t = ft_pitch(FT_TF32, hm);
+    const size_t t_bytes = (size_t)batch * 8 * hm * ld_t * (fmt == FT_EXT ? sizeof(float2) : sizeof(float));
     auto align = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
-    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, align(x_bytes) + align(w_bytes) + align(z_bytes), &st);
+    const size_t xb = align(ft_bytes(fmt, X)), wb = align(ft_bytes(fmt, W)), yb = align(ft_bytes(fmt, Y));
+    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, xb + wb + yb + t_bytes, &st);
     if (!work) return st;
-    TcOperand X{work, batch, nin, nin, ld};
-    TcOperand W{work + align(x_bytes), batch, nout, nin, ld};
-    TcOperand Z{work + align(x_bytes) + align(w_bytes), batch, nout, nin, ld};
-    void* c_d = coro::upload_async(ctx, c.data(), c.size() * sizeof(double), &st);
-    if (!c_d) return st;
-    std::vector<TcItem> it1(batch), it2(batch);
+    X.base = work;
+    W.base = work + xb;
+    Y.base = work + xb + wb;
+    void* T = work + xb + wb + yb;
+    std::vector<FtItem> items(batch);
+    for (int b = 0; b < batch; ++b) items[b] = FtItem{hn, hm, 0, b, -1, 0x7fffffff, 0, 1.0, 1.0};
+    std::vector<FtItem> both(items);
+    both.insert(both.end(), items.begin(), items.end());
     for (int b = 0; b < batch; ++b) {
-        it1[b] = TcItem{nin, nout, nin, b, b, 0, 0x7fffffff, 1.0f, 1.0f};
-        it2[b] = TcItem{nout, nout, nin, b, b, 0, 0x7fffffff, (float)c[b], 1.0f};
+        both[b].H = hn;                              // rows: k of the other axis, then u
+        both[batch + b].H = hm;
     }
-    void* i1 = coro::upload_async(ctx, it1.data(), batch * sizeof(TcItem), &st);
-    void* i2 = i1 ? coro::upload_async(ctx, it2.data(), batch * sizeof(TcItem), &st) : nullptr;
-    cudaError_t e = (i1 && i2) ? cudaSuccess : cudaErrorMemoryAllocation;
-    CUtensorMap mx, mw, mz;
-    if (e == cudaSuccess) e = tc_split(bf16, (const float2*)in->data, (long long)nin * nin, nin, X, ctx->stream);
-    if (e == cudaSuccess) e = tc_basis(bf16, (const double*)c_d, direction < 0 ? -1 : 1, W, ctx->stream);
-    if (e == cudaSuccess) e = tc_make_operand_map(X, bf16, &mx);
-    if (e == cudaSuccess) e = tc_make_operand_map(W, bf16, &mw);
-    if (e == cudaSuccess) e = tc_make_operand_map(Z, bf16, &mz);
+    std::vector<FtItem> plane(items);
+    for (int b = 0; b < batch; ++b) plane[b].scale = c[b];
+    both.insert(both.end(), plane.begin(), plane.end());
+    FtItem* it = (FtItem*)coro::upload_async(ctx, both.data(), both.size() * sizeof(FtItem), &st);
+    if (!it) return st;
+    FtGemm g1, g2;
+    cudaError_t e = ft_fold(fmt, (const float2*)in->data, (long long)n * n, n, n, hn, -1, X, ctx->stream);
+    for (int b = 0; b < batch && e == cudaSuccess; ++b) e = ft_basis(fmt, c[b], hn, hm, W, b, ctx->stream);
+    if (e == cudaSuccess) e = ft_make(fmt, X, W, batch, hm, 128, &g1);
+    if (e == cudaSuccess) e = ft_make(fmt, Y, W, batch, hm, 128, &g2);
     if (e == cudaSuccess) {
-        TcArgs a{};
-        a.items = (const TcItem*)i1;
+        FtArgs a{};
+        a.items = it;
         a.err = ctx->err;
-        a.dst = Z.base;
-        a.dst_bstride = (long long)4 * nout * ld;
-        a.dst_rows = nout;
-        a.dst_ld = ld;
-        e = tc_launch(bf16, TC_EPI_SPLITT, mx, mw, nin, nout, nin, batch, a, ctx->stream);
+        a.R = X.R;
+        a.dst = Y.base;
+        a.dst_bstride = Y.stride;
+        a.dst_R = Y.R;
+        a.dst_ld = Y.ld;
+        e = ft_launch(g1, FT_SPLIT, a, ctx->stream);
     }
     if (e == cudaSuccess) {
-        TcArgs a{};
-        a.items = (const TcItem*)i2;
+        FtArgs a{};
+        a.items = it + batch;
         a.err = ctx->err;
-        a.dst = out->data;
-        a.dst_bstride = (long long)nout * nout;
-        a.dst_rows = nout;
-        a.dst_ld = nout;
-        e = tc_launch(bf16, TC_EPI_C64T, mz, mw, nout, nout, nin, batch, a, ctx->stream);
+        a.R = Y.R;
+        a.dst = T;
+        a.dst_bstride = (long long)8 * hm * ld_t;
+        a.dst_R = hm;
+        a.dst_ld = ld_t;
+        e = ft_launch(g2, FT_FLOAT, a, ctx->stream);
     }
-    coro::free_async(ctx, c_d);
-    coro::free_async(ctx, i1);
-    coro::free_async(ctx, i2);
+    if (e == cudaSuccess) {
+        FtPlane p{};
+        p.items = it + 2 * batch;
+        p.T = T;
+        p.ext = fmt == FT_EXT;
+        p.R = hm;
+        p.ld = ld_t;
+        p.bstride = (long long)8 * hm * ld_t;
+        p.m = m;
+        p.sign = direction < 0 ? -1 : 1;
+        p.field = (float2*)out->data;
+        e = ft_plane(p, batch, ctx->stream);
+    }
+    coro::free_async(ctx, it);
     if (e == cudaErrorNotSupported) {
         coro::set_error("coro_propagate_mft: tensor maps unavailable (driver entry point missing)");
         return CORO_ENOTIMPL;
     }
     if (e != cudaSuccess) return coro::cuda_fail(e, "tensor-core MFT");
-    return CORO_OK;
-}
-
-// Extended-precision tensor-core MFT (CORO_MFT_EXT): the same two GEMMs on sliced BF16
-// operands (tcx_gemm.cu), the bases sliced straight from their FP64 values.
-coro_status mft_ext(coro_ctx ctx, const coro_wavefront* in, int direction, int m, const std::vector<double>& c,
-                    coro_wavefront* out) {
-    coro_status st = CORO_OK;
-    const int batch = in->batch;
-    const int nin = in->n, nout = m;
-    const int ld = tcx_ld(nin);
-    const size_t x_bytes = (size_t)TCX_X_PLANES * batch * nin * ld * 2;
-    const size_t w_bytes = (size_t)TCX_W_PLANES * batch * nout * ld * 2;
-    const size_t z_bytes = (size_t)TCX_X_PLANES * batch * nout * ld * 2;
-    auto align = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
-    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, align(x_bytes) + align(w_bytes) + align(z_bytes), &st);
-    if (!work) return st;
-    TcOperand X{work, batch, nin, nin, ld};
-    TcOperand W{work + align(x_bytes), batch, nout, nin, ld};
-    TcOperand Z{work + align(x_bytes) + align(w_bytes), batch, nout, nin, ld};
-    std::vector<TcItem> it1(batch), it2(batch);
-    for (int b = 0; b < batch; ++b) {
-        it1[b] = TcItem{nin, nout, nin, b, b, 0, 0x7fffffff, 1.0f, 1.0f};
-        it2[b] = TcItem{nout, nout, nin, b, b, 0, 0x7fffffff, (float)c[b], 1.0f};
-        it2[b].scale64 = c[b];
-    }
-    void* i1 = coro::upload_async(ctx, it1.data(), batch * sizeof(TcItem), &st);
-    void* i2 = i1 ? coro::upload_async(ctx, it2.data(), batch * sizeof(TcItem), &st) : nullptr;
-    cudaError_t e = (i1 && i2) ? cudaSuccess : cudaErrorMemoryAllocation;
-    // the first GEMM writes Z's nin valid columns only; its padding up to ld must read as zeros
-    if (e == cudaSuccess) e = cudaMemsetAsync(Z.base, 0, z_bytes, ctx->stream);
-    CUtensorMap mx, mw, mz;
-    if (e == cudaSuccess) e = tcx_split((const float2*)in->data, (long long)nin * nin, nin, X, ctx->stream);
-    for (int b = 0; b < batch && e == cudaSuccess; ++b)
-        e = tcx_basis_one(c[b], direction < 0 ? -1 : 1, W, b, nout, nin, ctx->stream);
-    if (e == cudaSuccess) e = tcx_make_x_map(X, &mx);
-    if (e == cudaSuccess) e = tcx_make_w_map(W, &mw);
-    if (e == cudaSuccess) e = tcx_make_x_map(Z, &mz);
-    if (e == cudaSuccess) {
-        TcArgs a{};
-        a.items = (const TcItem*)i1;
-        a.err = ctx->err;
-        a.dst = Z.base;
-        a.dst_bstride = (long long)TCX_X_PLANES * nout * ld;
-        a.dst_rows = nout;
-        a.dst_ld = ld;
-        e = tcx_launch(TC_EPI_SPLITT, mx, mw, nin, nout, batch, a, ctx->stream);
-    }
-    if (e == cudaSuccess) {
-        TcArgs a{};
-        a.items = (const TcItem*)i2;
-        a.err = ctx->err;
-        a.dst = out->data;
-        a.dst_bstride = (long long)nout * nout;
-        a.dst_rows = nout;
-        a.dst_ld = nout;
-        e = tcx_launch(TC_EPI_C64T, mz, mw, nout, nout, batch, a, ctx->stream);
-    }
-    coro::free_async(ctx, i1);
-    coro::free_async(ctx, i2);
-    if (e == cudaErrorNotSupported) {
-        coro::set_error("coro_propagate_mft: tensor maps unavailable (driver entry point missing)");
-        return CORO_ENOTIMPL;
-    }
-    if (e != cudaSuccess) return coro::cuda_fail(e, "extended-precision tensor-core MFT");
     return CORO_OK;
 }
 
@@ -236,9 +182,9 @@ extern "C" coro_status coro_propagate_mft(coro_ctx ctx, const coro_wavefront* in
         c[b] = du[b] / npix;
     }
     coro::DeviceGuard g(ctx->device);
-    if (precision == CORO_MFT_EXT) return mft_ext(ctx, in, direction, m, c, out);
+    if (precision == CORO_MFT_EXT) return mft_tensor_core(ctx, in, direction, m, c, FT_EXT, out);
     if (precision == CORO_MFT_3XTF32 || precision == CORO_MFT_3XBF16)
-        return mft_tensor_core(ctx, in, direction, m, c, precision == CORO_MFT_3XBF16, out);
+        return mft_tensor_core(ctx, in, direction, m, c, precision == CORO_MFT_3XBF16 ? FT_BF16 : FT_TF32, out);
     return dbl ? mft_cuda_cores<double2>(ctx, in, direction, m, c, out) : mft_cuda_cores<float2>(ctx, in, direction, m, c, out);
 }
 

@@ -130,6 +130,18 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
     return d;
 }
 
+// The same for the 128-byte swizzle: rows of 128 bytes, 8-row (1024-byte) atoms; a K step of 32
+// bytes moves the start address inside the row.
+__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;                            // layout: 128-byte swizzle
+    return d;
+}
+
 // Instruction descriptor (kind::tf32 or kind::f16 with BF16 inputs), FP32 accumulate,
 // both operands K-major, M x N tile; negA flips the sign of A.
 template <bool BF16>
@@ -159,28 +171,29 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, ui
     }
 }
 
-// BF16 MMA with the A-operand collector: FILL reads A from shared memory and keeps it; USE
+// MMA with the A-operand collector: FILL reads A from shared memory and keeps it; USE
 // takes A from the collector (a previous FILL with the same descriptor, no MMA with another A
 // in between); LASTUSE does the same and releases it. Consecutive MMAs that share A then
 // read it from shared memory once.
 enum CollectorOp { COLL_NONE = 0, COLL_FILL = 1, COLL_USE = 2, COLL_LASTUSE = 3 };
+#define CORO_UMMA_COLL(KIND, OPNAME)                                                              \
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"                               \
+                 "tcgen05.mma.cta_group::1.kind::" KIND ".collector::a::" OPNAME " [%0], %1, %2, %3, p;\n\t}\n" \
+                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(id), "r"(acc) : "memory")
+template <bool BF16, int OP>
+__device__ __forceinline__ void umma_coll(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+    if constexpr (OP == COLL_NONE) umma<BF16>(d_tmem, a, b, id, acc);
+    else if constexpr (BF16 && OP == COLL_FILL) CORO_UMMA_COLL("f16", "fill");
+    else if constexpr (BF16 && OP == COLL_USE) CORO_UMMA_COLL("f16", "use");
+    else if constexpr (BF16) CORO_UMMA_COLL("f16", "lastuse");
+    else if constexpr (OP == COLL_FILL) CORO_UMMA_COLL("tf32", "fill");
+    else if constexpr (OP == COLL_USE) CORO_UMMA_COLL("tf32", "use");
+    else CORO_UMMA_COLL("tf32", "lastuse");
+}
+#undef CORO_UMMA_COLL
 template <int OP>
 __device__ __forceinline__ void umma_bf16_coll(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
-    if constexpr (OP == COLL_FILL) {
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}\n"
-                     ::"r"(d_tmem), "l"(a), "l"(b), "r"(id), "r"(acc) : "memory");
-    } else if constexpr (OP == COLL_USE) {
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}\n"
-                     ::"r"(d_tmem), "l"(a), "l"(b), "r"(id), "r"(acc) : "memory");
-    } else if constexpr (OP == COLL_LASTUSE) {
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}\n"
-                     ::"r"(d_tmem), "l"(a), "l"(b), "r"(id), "r"(acc) : "memory");
-    } else {
-        umma<true>(d_tmem, a, b, id, acc);
-    }
+    umma_coll<true, OP>(d_tmem, a, b, id, acc);
 }
 
 // Arrive on `bar` once every previously issued MMA of this thread has completed.

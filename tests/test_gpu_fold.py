@@ -69,3 +69,46 @@ def test_lyot_halves(ctx, n, npix, frac, m_occ, spot, m_det, prec, tol):
         det = coronagraph.lyot_fields(xs[b], p)["det"]
         assert np.max(np.abs(fld[b].cpu().numpy() - det)) < 30 * (tol + 6e-8) * np.abs(det).max()
     plan.close()
+
+
+# masks inside their arrays (parity classes) and reaching unpaired edges (complex GEMMs); both dark
+# holes end inside the detector, or the second one's reaches its unpaired edge
+TC_CASES = [(64, 60.0, 0.8, 32, 3.0, 48, 11.0), (65, 65.0, 0.9, 33, 3.9, 47, 10.0), (130, 130.0, 0.99, 40, 2.0, 50, 11.0),
+            (131, 120.0, 0.7, 39, 0.0, 129, 11.0), (257, 240.0, 0.8, 64, 7.0, 131, 25.0), (300, 300.0, 0.5, 33, 1.0, 290, 30.0),
+            (64, 64.0, 1.0, 32, 3.0, 48, 11.0), (64, 60.0, 0.8, 32, 4.0, 48, 11.0), (64, 60.0, 0.8, 32, 3.0, 48, 12.0)]
+
+
+@pytest.mark.parametrize("prec", [coro.MFT_3XTF32, coro.MFT_3XBF16, coro.MFT_EXT])
+@pytest.mark.parametrize("n,npix,frac,m_occ,spot,m_det,dh_out", TC_CASES)
+def test_lyot_tensor_core_halves(ctx, n, npix, frac, m_occ, spot, m_det, dh_out, prec):
+    """Image, peak, field, dark-hole sum and adjoint at the bars of the batched Lyot tests (whole
+    image 1e-5 of the peak; peak 1e-5, extended 1e-9; adjoint 1e-3)."""
+    from oracle import adjoint
+    lam = 550e-9
+    items = [dict(m_occ=m_occ, du_occ=0.25, spot_radius=spot, du_det=0.5, dh_in=4.0, dh_out=dh_out),
+             dict(m_occ=m_occ + 1, du_occ=0.27, spot_radius=spot, du_det=0.45, dh_in=3.0, dh_out=0.85 * dh_out)]
+    ph = np.exp(1j * inputs.rng(n).uniform(-0.2, 0.2, (2, n, n)))
+    pupil = np.stack([coronagraph.pupil_field(n, npix, lam, None) * p for p in ph]).astype(np.complex64)
+    x = torch.from_numpy(pupil).cuda()
+    plan = coro.LyotPlan(ctx, n=n, npix=npix, lyot_frac=frac, m_det=m_det, items=items, precision=prec)
+    peak = plan.peak(x)
+    img = torch.empty((2, m_det, m_det), dtype=torch.float32, device="cuda")
+    fld = torch.empty((2, m_det, m_det), dtype=torch.complex64, device="cuda")
+    dh = plan.execute(x, peak=peak, intensity=img, field=fld)
+    g, dh_g = plan.gradient(x, peak)
+    again = torch.empty_like(img)
+    plan.execute(x, peak=peak, intensity=again)          # the gradient leaves nothing behind
+    assert torch.equal(img, again)
+    for b, it in enumerate(items):
+        p = coronagraph.LyotParams(n, npix, it["m_occ"], it["du_occ"], it["spot_radius"], frac, m_det, it["du_det"])
+        e = pupil[b].astype(np.complex128)
+        ref, s, pk = coronagraph.lyot_psf(e, p, it["dh_in"], it["dh_out"])
+        mask = coronagraph.dark_hole_mask(m_det, it["du_det"], it["dh_in"], it["dh_out"])
+        assert abs(peak[b] / pk - 1) < (1e-9 if prec == coro.MFT_EXT else 1e-5)
+        assert np.max(np.abs(img[b].cpu().numpy() - ref)) < 1e-5
+        assert abs(dh[b] - s) < 1e-3 * s + mask.sum() * 1e-7
+        assert abs(dh_g[b] - s) < 1e-3 * s + mask.sum() * 1e-7
+        det = coronagraph.lyot_fields(e, p)["det"]
+        assert rel_l2(fld[b].cpu().numpy(), det) < 1e-3
+        assert rel_l2(g[b].cpu().numpy(), adjoint.lyot_adjoint(mask * det / pk, p)) < 1e-3
+    plan.close()
