@@ -320,9 +320,12 @@ coro_status coro_fresnel_plan_set_pass_kernel(coro_plan plan, int row_variant, i
  * ([b][x][y], contiguous rows) into a plane the plan owns (batch x n x n complex64, allocated
  * here, freed on return to 0 or with the plan), and the row pass reads it back column-wise
  * and writes the field's rows; each pass then has one strided side. Results agree up to FP32
- * rounding order. At creation the plan times both and keeps the faster (natural when
- * CORO_AUTOTUNE=0) unless the environment sets CORO_LAYOUT=0 (natural) or CORO_LAYOUT=1
- * (alternating). CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a
+ * rounding order. A plan starts on neither: at creation it takes the natural passes its tuner
+ * picked, or (when faster, and without tuning) the packed-pair kernels with row pairs held
+ * sample by sample interleaved between passes, in place, reported as layout 0; results are
+ * bitwise those of the same kernels on the natural layout. The environment sets CORO_LAYOUT=0
+ * to keep natural rows throughout, CORO_LAYOUT=1 for the alternating layout.
+ * CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a
  * supported size. */
 coro_status coro_fresnel_plan_set_layout(coro_plan plan, int transposed);
 /* Give dst the kernel choices and layout the tuner made for src (plans of the same dtype, n,

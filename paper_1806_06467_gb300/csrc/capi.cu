@@ -616,6 +616,28 @@ struct Op {
     int variant = -1;     // row passes: -1 default, 0 persistent, 1 per group, 2 units, 3 pairs
 };
 
+// Interleaved row pairs (complex64, n = 1024 ... 4096): between a row pass and the next the field
+// holds rows 2m and 2m + 1 sample by sample, which halves the rows that the column pass's strided
+// copies are made of (col_pass_pair_kernel). Every column pass between two row passes takes that
+// form, all passes on the packed-pair kernels; what enters and leaves the plan, and a column pass
+// that ends it, stay natural. nat: the same passes on the same kernels in the natural layout, whose
+// results are bitwise equal. Returns the number of such column passes.
+int interleaved_ops(int dtype, int n, std::vector<Op>& nat, std::vector<Op>* out) {
+    if (dtype != CORO_C64 || n < 1024 || n > 4096 || (n & (n - 1))) return 0;
+    int found = 0;
+    for (size_t i = 1; i + 1 < nat.size(); ++i) found += !nat[i].row && nat[i - 1].row && nat[i + 1].row;
+    if (!found) return 0;
+    for (Op& op : nat) (op.row ? op.variant : op.lines) = op.row ? 3 : -3;
+    *out = nat;
+    for (size_t i = 1; i + 1 < nat.size(); ++i) {
+        if (nat[i].row || !nat[i - 1].row || !nat[i + 1].row) continue;
+        (*out)[i].lines = -9;
+        (*out)[i - 1].row_flags |= RF_OUT_IL;
+        (*out)[i + 1].row_flags |= RF_IN_IL;
+    }
+    return found;
+}
+
 // ev (optional, ops.size() + 1 events): recorded before the first pass and after each.
 // tbuf: the plane that column passes with lines -6 write transposed and the row passes of
 // variant 4 read back (batch x n x n samples); NULL when the ops hold neither.
@@ -845,6 +867,8 @@ extern "C" coro_status coro_propagate_fresnel(coro_ctx ctx, coro_wavefront* wf, 
             }
         }
     }
+    std::vector<Op> il;
+    if (st == CORO_OK && interleaved_ops(wf->dtype, n, ops, &il)) ops = il;
     if (st == CORO_OK) st = run_ops_any(ctx, wf->dtype, n, batch, ops, wf->data);
     db.release();
     if (st == CORO_OK && method == CORO_FRESNEL_DIRECT)
@@ -995,6 +1019,7 @@ struct FresnelPlan : coro_plan_s {
     std::vector<Op> ops;             // as executed
     std::vector<Op> ops_nat;         // the same passes, every one in place on the natural layout
     void* tbuf = nullptr;            // transposed plane of the alternating layout (owned)
+    bool interleaved = false;        // ops run on interleaved row pairs (interleaved_ops)
     DevBlocks db;
     std::vector<double> ps_final;
     std::vector<std::string> tune_log;
@@ -1059,6 +1084,7 @@ coro_status set_layout(FresnelPlan* p, int transposed) {
             p->tbuf = nullptr;
         }
     }
+    p->interleaved = false;
     p->graph.reset();                                   // a captured graph holds the old kernels
     return CORO_OK;
 }
@@ -1178,27 +1204,34 @@ coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0,
     return CORO_OK;
 }
 
-// Layout choice: CORO_LAYOUT=0 / 1 forces the natural / alternating layout; otherwise the
-// alternating one is timed against the natural one when tuning is on and kept if faster
-// (natural without tuning).
+// Layout choice: CORO_LAYOUT=0 / 1 forces the natural / alternating layout; otherwise interleaved
+// row pairs, unless tuning is on and finds the tuned natural passes faster. (Alternating has not
+// been the fastest anywhere: 965 us against 846 natural for the 4096^2 relay; it is there for
+// coro_fresnel_plan_set_layout.)
 void choose_layout(FresnelPlan* p) {
-    if (transposed_ops(p->dtype, p->n, p->ops_nat, nullptr) == 0) return;
     const char* v = std::getenv("CORO_LAYOUT");
-    const bool force = v && v[0] == '1';
-    if ((v && v[0] == '0') || (!force && !autotune_enabled())) return;
-    if (set_layout(p, 1) != CORO_OK) { clear_error(); return; }     // no room: natural layout
-    if (force) return;
-    coro_status st = CORO_OK;
-    const size_t bytes = (size_t)p->batch * p->n * p->n * sizeof(float2);
-    void* scratch = upload_async(p->ctx, nullptr, bytes, &st);
-    if (!scratch) { clear_error(); return; }
-    cudaMemsetAsync(scratch, 0, bytes, p->ctx->stream);
-    const float t_nat = time_ops<float2>(p->ctx, p->n, p->batch, timing_copy(p->ops_nat), scratch, 3);
-    const float t_alt = time_ops<float2>(p->ctx, p->n, p->batch, timing_copy(p->ops), scratch, 3, p->tbuf);
-    free_async(p->ctx, scratch);
-    p->tune_log.push_back("layout natural: " + std::to_string(t_nat / 3) + " ms, alternating: " +
-                          std::to_string(t_alt / 3) + " ms");
-    if (!(t_alt < t_nat)) set_layout(p, 0);
+    if (v && v[0] == '0') return;
+    if (v && v[0] == '1') {
+        if (transposed_ops(p->dtype, p->n, p->ops_nat, nullptr) && set_layout(p, 1) != CORO_OK) clear_error();   // no room: natural
+        return;
+    }
+    std::vector<Op> nat = p->ops_nat, il;
+    if (!interleaved_ops(p->dtype, p->n, nat, &il)) return;
+    if (autotune_enabled()) {
+        coro_status st = CORO_OK;
+        const size_t bytes = (size_t)p->batch * p->n * p->n * sizeof(float2);
+        void* scratch = upload_async(p->ctx, nullptr, bytes, &st);
+        if (!scratch) { clear_error(); return; }
+        cudaMemsetAsync(scratch, 0, bytes, p->ctx->stream);
+        const float t_nat = time_ops<float2>(p->ctx, p->n, p->batch, timing_copy(p->ops_nat), scratch, 3);
+        const float t_il = time_ops<float2>(p->ctx, p->n, p->batch, timing_copy(il), scratch, 3);
+        free_async(p->ctx, scratch);
+        p->tune_log.push_back("layout natural: " + std::to_string(t_nat / 3) + " ms, interleaved: " + std::to_string(t_il / 3) + " ms");
+        if (!(t_il < t_nat)) return;
+    }
+    p->ops_nat = nat;
+    p->ops = il;
+    p->interleaved = true;
 }
 
 coro_status finish_plan(coro_ctx ctx, std::unique_ptr<FresnelPlan>& plan, coro_plan* out, const char* who) {
@@ -1561,6 +1594,7 @@ extern "C" coro_status coro_fresnel_plan_copy_tuning(coro_plan dst, coro_plan sr
     d->ops = d->ops_nat;
     coro_status st = set_layout(d, 0);
     if (st == CORO_OK && s->tbuf) st = set_layout(d, 1);
+    if (st == CORO_OK && s->interleaved) d->interleaved = interleaved_ops(d->dtype, d->n, d->ops_nat, &d->ops) > 0;
     return st;
 }
 

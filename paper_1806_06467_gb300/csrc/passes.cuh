@@ -513,7 +513,9 @@ __device__ __forceinline__ void apply_elems_pair(pk::CP (&v)[16], int x0, int ya
 enum RowFlags : int {
     RF_INV_FIRST = 1,     // inverse row FFT before the elements
     RF_FWD_AFTER = 2,     // forward row FFT after the elements
-    RF_INIT_ONE = 4       // do not read: the field starts as 1 + 0i
+    RF_INIT_ONE = 4,      // do not read: the field starts as 1 + 0i
+    RF_IN_IL = 8,         // packed-pair kernel only: rows 2m and 2m + 1 are read, or
+    RF_OUT_IL = 16        // written, sample by sample interleaved (see col_pass_pair_kernel)
 };
 
 template <typename C>
@@ -930,14 +932,25 @@ template <int N, int U, int S> struct PColPairCfg {
 
 // TOUT: the pair leaves as two contiguous rows of the transposed plane out[b][x][y] (one bulk
 // store of 2N samples) instead of two strided columns of out[b][y][x]; out must not alias in.
-template <int N, int U, int S, bool TOUT>
+//
+// IL: the field holds rows 2m and 2m + 1 sample by sample interleaved, [b][m][x][2], as the row
+// passes before and after this one write and read it (their two rows are the same 16 N contiguous
+// bytes in either form, and so are the strip's bytes here: every pass stays in place). A column
+// pair of a row pair is then one whole 32-byte sector instead of two halves of two, and the strip
+// N/2 box rows of 32 bytes instead of N of 16. The copy engine's rate is in box rows (about 1.7
+// clocks each over loads and stores), which is what held the natural form: 4096^2 95 -> 80 us,
+// 5 x 2048^2 likewise. (One-line kernels on this layout, lanes alternating between the two rows:
+// columns 108 / 129 us, rows 89 us against 83; not kept.)
+// The boxes use the 32-byte swizzle: 16-byte halves swapped in every second group of four row pairs,
+// which spreads the samples of one column that 16 threads read over all banks.
+template <int N, int U, int S, bool TOUT, bool IL>
 __global__ void __launch_bounds__(PColPairCfg<N, U, S>::THREADS, 1)
 col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_constant__ CUtensorMap map, int groups) {
     using Cfg = PColPairCfg<N, U, S>;
     using pk::CP;
     constexpr uint32_t BYTES = Cfg::GROUP * sizeof(float2);
     constexpr int GPI = N / 2;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
     float2* stage = reinterpret_cast<float2*>(smem_raw);
     const int u = threadIdx.x / Cfg::UT;
     const int t = threadIdx.x % Cfg::UT;
@@ -947,6 +960,10 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
     const SyncNamed sync{1 + u, Cfg::UT};
     const bool leader = t == 0;
     const float2* tw = a.tw;
+    static_assert(!(TOUT && IL), "one output form");
+    static_assert(!IL || (Cfg::REGION * sizeof(float2) % 256 == 0 && Cfg::TPL % 16 == 0), "swizzle atoms of 256 bytes");
+    // IL: column A's sample of row t (of t + s TPL: s 2 TPL samples on) and column B's
+    const int half = (t >> 3) & 1, il_a = (t >> 1) * 4 + half * 2 + (t & 1), il_b = il_a + (half ? -2 : 2);
 
     auto issue_load = [&](int k) {
         const int g = blockIdx.x + k * gridDim.x;
@@ -955,7 +972,10 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
         uint64_t* bar = &full[k % U];
         tc::mbar_arrive_expect_tx(bar, BYTES);
 #pragma unroll 1
-        for (int q = 0; q < Cfg::BOXES; ++q) tc::tma_load_2d(dst + q * 512, &map, bar, x, y + q * 256);
+        for (int q = 0; q < (IL ? N / 512 : Cfg::BOXES); ++q) {
+            if constexpr (IL) tc::tma_load_2d(dst + q * 1024, &map, bar, 2 * x, y / 2 + q * 256);
+            else tc::tma_load_2d(dst + q * 512, &map, bar, x, y + q * 256);
+        }
     };
     const int mine = groups > (int)blockIdx.x ? (groups - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (threadIdx.x == 0) {
@@ -973,10 +993,19 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
         const float4* src = reinterpret_cast<const float4*>(stage + (k % S) * Cfg::GROUP);
         if (ok) ok = tc::mbar_wait(&full[u], j & 1, a.err, 9);
         CP v[16];
+        if constexpr (IL) {
+            const float2* src2 = stage + (k % S) * Cfg::GROUP;
 #pragma unroll
-        for (int s = 0; s < 16; ++s) {
-            const float4 q = src[t + s * Cfg::TPL];       // row t + s*TPL: (re_A, im_A, re_B, im_B)
-            v[s] = CP{pk::pack(q.x, q.z), pk::pack(q.y, q.w)};
+            for (int s = 0; s < 16; ++s) {
+                const float2 qa = src2[il_a + s * 2 * Cfg::TPL], qb = src2[il_b + s * 2 * Cfg::TPL];
+                v[s] = CP{pk::pack(qa.x, qb.x), pk::pack(qa.y, qb.y)};
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < 16; ++s) {
+                const float4 q = src[t + s * Cfg::TPL];       // row t + s*TPL: (re_A, im_A, re_B, im_B)
+                v[s] = CP{pk::pack(q.x, q.z), pk::pack(q.y, q.w)};
+            }
         }
         if (leader) tc::bulk_wait_read<0>();
         sync();
@@ -1008,6 +1037,15 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
                 region[t + s * Cfg::TPL] = qa;
                 region[N + t + s * Cfg::TPL] = qb;
             }
+        } else if constexpr (IL) {
+#pragma unroll
+            for (int s = 0; s < 16; ++s) {
+                float2 qa, qb;
+                pk::unpack(v[s].re, qa.x, qb.x);
+                pk::unpack(v[s].im, qa.y, qb.y);
+                region[il_a + s * 2 * Cfg::TPL] = qa;
+                region[il_b + s * 2 * Cfg::TPL] = qb;
+            }
         } else {
             float4* out = reinterpret_cast<float4*>(region);
 #pragma unroll
@@ -1023,6 +1061,9 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
         if (leader) {
             if constexpr (TOUT) {
                 tc::bulk_store(a.out + ((size_t)b * N + col) * N, region, BYTES);
+            } else if constexpr (IL) {
+#pragma unroll 1
+                for (int q = 0; q < N / 512; ++q) tc::tma_store_2d(&map, region + q * 1024, 2 * col, b * (N / 2) + q * 256);
             } else {
                 const int x = col, y = b * N;
 #pragma unroll 1
@@ -1407,7 +1448,7 @@ row_pass_pair_kernel(const __grid_constant__ RowArgs<float2> a, const __grid_con
         if (load) {
             const float2* src = stage + (k % S) * Cfg::GROUP;
             if (ok) ok = tc::mbar_wait(&full[u], j & 1, a.err, 11);
-            if constexpr (TIN) {
+            if (TIN || (a.flags & RF_IN_IL)) {
                 const float4* src4 = reinterpret_cast<const float4*>(src);
 #pragma unroll
                 for (int s = 0; s < 16; ++s) {
@@ -1432,13 +1473,24 @@ row_pass_pair_kernel(const __grid_constant__ RowArgs<float2> a, const __grid_con
         if (a.flags & RF_INV_FIRST) pk::line_fft2<N, true>(v, xl, t, a.tw, sync);
         if (a.elems.count) apply_elems_pair<N, Cfg::TPL>(v, t, ya, b, a.elems);
         if (a.flags & RF_FWD_AFTER) pk::line_fft2<N, false>(v, xl, t, a.tw, sync);
+        if (a.flags & RF_OUT_IL) {
+            float4* out = reinterpret_cast<float4*>(region);
 #pragma unroll
-        for (int s = 0; s < 16; ++s) {
-            float2 qa, qb;
-            pk::unpack(v[s].re, qa.x, qb.x);
-            pk::unpack(v[s].im, qa.y, qb.y);
-            region[t + s * Cfg::TPL] = qa;
-            region[N + t + s * Cfg::TPL] = qb;
+            for (int s = 0; s < 16; ++s) {
+                float4 q;
+                pk::unpack(v[s].re, q.x, q.z);
+                pk::unpack(v[s].im, q.y, q.w);
+                out[t + s * Cfg::TPL] = q;
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < 16; ++s) {
+                float2 qa, qb;
+                pk::unpack(v[s].re, qa.x, qb.x);
+                pk::unpack(v[s].im, qa.y, qb.y);
+                region[t + s * Cfg::TPL] = qa;
+                region[N + t + s * Cfg::TPL] = qb;
+            }
         }
         tc::fence_proxy_async();
         sync();

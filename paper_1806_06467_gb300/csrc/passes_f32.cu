@@ -46,7 +46,7 @@ cudaError_t launch_row_pass<float2>(int n, const RowArgs<float2>& a, const PassL
 // -2 = unit-pipelined kernel (two columns per unit), -3 = unit-pipelined kernel on packed
 // FP32x2 column pairs, -4 = wide kernel (four columns, packed pairs, staged by TMA), -6 = the
 // packed-pair kernel writing its result transposed to a separate plane (row variant 4 reads it),
-// -7 = quad kernel (four columns as two packed pairs, whole-sector strips, swizzled exchanges),
+// -9 = the packed-pair kernel on interleaved row pairs (plans only, see interleaved_ops), -7 = quad kernel (four columns as two packed pairs, whole-sector strips, swizzled exchanges),
 // -8 = the shared-memory Stockham engine of mixed.cuh with radix 8 (N = 8^k x 2 or 4): the
 // alternative factorisation of the power-of-two lengths; mixed-radix lengths: columns per block
 // of the shared-memory engine, or -5 = the packed-pair engine of mixed_pair.cuh (its lengths).
@@ -65,6 +65,7 @@ cudaError_t launch_col_pass<float2>(int n, int lines, const ColArgs<float2>& a, 
             if (lines == -7) return col_launch_quad<1024>(a, l);
             if (lines == -4) return col_launch_wide<1024>(a, l);
             if (lines == -6) return col_launch_pair<1024, 8, 4, true>(a, l);
+            if (lines == -9) return col_launch_pair<1024, 8, 4, false, true>(a, l);
             if (lines == -3) return col_launch_pair<1024, 8, 4>(a, l);
             if (lines == -2) return col_launch_units<float2, 1024, 2, 8, 4>(a, l);
             if (lines == -1) return col_launch_persistent<float2, 1024, 4>(a, l);
@@ -74,6 +75,7 @@ cudaError_t launch_col_pass<float2>(int n, int lines, const ColArgs<float2>& a, 
             if (lines == -7) return col_launch_quad<2048>(a, l);
             if (lines == -4) return col_launch_wide<2048>(a, l);
             if (lines == -6) return col_launch_pair<2048, 4, 2, true>(a, l);
+            if (lines == -9) return col_launch_pair<2048, 4, 2, false, true>(a, l);
             if (lines == -3) return col_launch_pair<2048, 4, 2>(a, l);
             if (lines == -2) return col_launch_units<float2, 2048, 2, 4, 2>(a, l);
             if (lines == -1) return col_launch_persistent<float2, 2048, 2>(a, l);
@@ -83,6 +85,7 @@ cudaError_t launch_col_pass<float2>(int n, int lines, const ColArgs<float2>& a, 
             if (lines == -7) return col_launch_quad<4096>(a, l);
             if (lines == -4) return col_launch_wide<4096>(a, l);
             if (lines == -6) return col_launch_pair<4096, 2, 1, true>(a, l);
+            if (lines == -9) return col_launch_pair<4096, 2, 1, false, true>(a, l);
             if (lines == -3) return col_launch_pair<4096, 2, 1>(a, l);
             if (lines == -2) return col_launch_units<float2, 4096, 2, 2, 1>(a, l);
             if (lines == -1) return col_launch_persistent<float2, 4096, 2>(a, l);
@@ -179,6 +182,7 @@ bool mixed_length_ok(int n, bool dbl) { return dbl ? mixed_supported<double2>(n)
 
 void describe_pass(int n, bool dbl, bool row, int variant, int lines, int* persistent, int* out_lines) {
     int p = 0, w = 0;
+    if (lines == -9) lines = -3;                            // packed column pairs of interleaved row pairs
     if ((n & (n - 1)) && !dbl) {                            // the defaults of launch_*_pass<float2>
         if (row && variant < 0) variant = row_variant_default(n);
         if (!row && lines == 0) lines = col_lines_default(n, false);

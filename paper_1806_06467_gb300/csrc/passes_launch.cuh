@@ -126,22 +126,24 @@ cudaError_t col_launch_units(const ColArgs<C>& a, const PassLaunch& l) {
     return cudaGetLastError();
 }
 
-// TOUT: out-of-place, the result transposed (out[b][x][y]).
-template <int N, int U, int S, bool TOUT = false>
+// TOUT: out-of-place, the result transposed (out[b][x][y]). IL: row pairs interleaved ([b][m][x][2]).
+template <int N, int U, int S, bool TOUT = false, bool IL = false>
 cudaError_t col_launch_pair(const ColArgs<float2>& a, const PassLaunch& l) {
     using Cfg = PColPairCfg<N, U, S>;
     static unsigned done = 0;
     const size_t smem = Cfg::template smem<float2>();
-    cudaError_t e = ensure_smem(col_pass_pair_kernel<N, U, S, TOUT>, smem, done);
+    cudaError_t e = ensure_smem(col_pass_pair_kernel<N, U, S, TOUT, IL>, smem, done);
     if (e != cudaSuccess) return e;
     int sms = 0;
     if ((e = sm_count(&sms)) != cudaSuccess) return e;
     if ((a.in != a.out) != TOUT) return cudaErrorInvalidValue;
     CUtensorMap map;
-    if ((e = tc_make_field_map(a.in, N, (long long)l.batch * N, 2, &map)) != cudaSuccess) return e;
+    e = IL ? tc_make_field_map(a.in, 2 * N, (long long)l.batch * N / 2, 4, &map, 256, true)
+           : tc_make_field_map(a.in, N, (long long)l.batch * N, 2, &map);
+    if (e != cudaSuccess) return e;
     const int groups = l.batch * N / 2;
     const int grid = groups < sms ? groups : sms;
-    col_pass_pair_kernel<N, U, S, TOUT><<<grid, Cfg::THREADS, smem, l.stream>>>(a, map, groups);
+    col_pass_pair_kernel<N, U, S, TOUT, IL><<<grid, Cfg::THREADS, smem, l.stream>>>(a, map, groups);
     return cudaGetLastError();
 }
 

@@ -402,7 +402,7 @@ cudaError_t tc_make_operand_map(const TcOperand& op, bool bf16, CUtensorMap* map
 }
 
 cudaError_t tc_make_field_map(const void* base, int n, long long rows_total, int box_cols, CUtensorMap* map,
-                              int box_rows) {
+                              int box_rows, bool swizzle32) {
     auto fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
     if (((uintptr_t)base & 15) || box_cols * 8 % 16 || box_rows < 1 || box_rows > 256 || rows_total < box_rows)
@@ -412,8 +412,8 @@ cudaError_t tc_make_field_map(const void* base, int n, long long rows_total, int
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 

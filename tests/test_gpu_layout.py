@@ -210,3 +210,37 @@ def test_pass_flops(ctx):
     f = [plan.pass_flops(i) for i in range(plan.launch_count)]
     assert f[0] == one and f[-1] == one
     assert all(x == 2 * one for x in f[1:-1])
+
+
+@pytest.mark.parametrize("n,batch", [(1024, 3), (2048, 2), (4096, 1)])
+def test_interleaved_row_pairs_match_natural_layout(ctx, n, batch):
+    """A plan as created untuned (row pairs interleaved between passes), with a checkpoint, a direct
+    hop of each sign, is bitwise the same kernels on the natural layout."""
+    import os
+    from oracle import propagation
+    lam = np.linspace(500e-9, 600e-9, batch)
+    dx, z = 1.0 / n, [1.5, 40.0, -3.0, 2.0]
+    meth = [coro.FRESNEL_AS, coro.FRESNEL_DIRECT, coro.FRESNEL_DIRECT, coro.FRESNEL_AS]
+    f = inputs.random_field((batch, n, n), seed=n).astype(np.complex64)
+    out, stored = [], []
+    for env in ({"CORO_AUTOTUNE": "0"}, {"CORO_AUTOTUNE": "0", "CORO_LAYOUT": "0"}):
+        store = torch.zeros((batch, n, n), dtype=torch.complex64, device="cuda")
+        els = [coro.element(coro.EL_APERTURE, plane=0, radius=0.3), coro.element(coro.EL_CHECKPOINT, plane=1, store=store),
+               coro.element(coro.EL_LENS, plane=3, focal_length=7.0)]
+        old = {k: os.environ.get(k) for k in env}
+        os.environ.update(env)
+        try:
+            plan = coro.FresnelPlan(ctx, n=n, batch=batch, pixelscale=dx, wavelength=lam, distances=z, methods=meth, elements=els)
+        finally:
+            for k, v in old.items():
+                os.environ.pop(k) if v is None else os.environ.__setitem__(k, v)
+        x = torch.from_numpy(f).cuda()
+        plan.execute(x)
+        out.append(x)
+        stored.append(store)
+        assert not plan.layout
+    assert torch.equal(out[0], out[1]) and torch.equal(stored[0], stored[1])
+    if n == 1024:                                        # and against the oracle through the first hop
+        from oracle import optics
+        ref = propagation.angular_spectrum(f[0] * optics.circular_aperture(n, dx, 0.3), dx, lam[0], z[0])
+        assert np.linalg.norm(stored[0][0].cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
