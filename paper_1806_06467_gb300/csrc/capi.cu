@@ -480,7 +480,7 @@ void split_f32(double x, float* hi, float* lo) {
 
 // Compile one API element for a batch at the given per-item pixel scales.
 coro_status compile_element(DevBlocks& db, const coro_element* el, bool dbl, int n, int batch,
-                            const double* ps, const double* lam, DevElem* out) {
+                            const double* ps, const double* lam, DevElem* out, bool own = false) {
     coro_status st = CORO_OK;
     std::memset(out, 0, sizeof(DevElem));
     std::vector<int> ithr((size_t)batch * 4, 0);
@@ -517,7 +517,8 @@ coro_status compile_element(DevBlocks& db, const coro_element* el, bool dbl, int
         }
         case CORO_EL_OPD_MAP: {
             if (!el->opd) { set_error("opd map: opd pointer is NULL"); return CORO_EINVAL; }
-            for (int b = 0; b < batch; ++b) split_f32(2.0 / lam[b], &fpar[4 * b], &fpar[4 * b + 1]);
+            const double sign = own && (el->flags & kElfMapNegate) ? -1.0 : 1.0;
+            for (int b = 0; b < batch; ++b) split_f32(sign * 2.0 / lam[b], &fpar[4 * b], &fpar[4 * b + 1]);
             out->kind = DK_OPD_MAP;
             out->map = el->opd;
             out->amp = el->amplitude;
@@ -612,6 +613,13 @@ struct Op {
     PassElems elems{};
     const void* tab_x = nullptr;
     const void* tab_y = nullptr;
+    // rows that a mask of this (row) pass leaves: n/2 - mask_r ... n/2 + mask_r; -1: no mask. mask_map /
+    // mask_store: a map after the mask (its infinities would leave the mask), an element that writes
+    // to caller memory
+    int mask_r = -1;
+    bool mask_map = false, mask_store = false;
+    // the rows and boxes that the pass runs (RowArgs, ColArgs); hi = 0: all
+    int row_lo = 0, row_hi = 0, in_lo = 0, in_hi = 0, out_lo = 0, out_hi = 0;
     int lines = 0;        // column passes: 0 default, > 0 block width, < 0 staged kernels (passes_f32.cu)
     int variant = -1;     // row passes: -1 default, 0 persistent, 1 per group, 2 units, 3 pairs
 };
@@ -636,6 +644,41 @@ int interleaved_ops(int dtype, int n, std::vector<Op>& nat, std::vector<Op>* out
         (*out)[i + 1].row_flags |= RF_IN_IL;
     }
     return found;
+}
+
+// Rows that cannot matter are left out of interleaved passes: behind a mask (an aperture or stop) only
+// the rows it leaves are transformed, written before it by the column pass and read after it by the
+// next one, in boxes of 256 rows; a plan's last row pass fills its other rows with zeros. first_in: rows
+// n/2 +- first_in are all the input's non-zeros (-1: unknown); last_out: only rows n/2 +- last_out of the
+// result are wanted (-1: all; the others are then left as they are). The first plane's mask counts
+// where the plan makes the field itself (INIT_ONE), so that what a caller's field holds under the mask
+// reaches the passes as before. Skipped are products with zeros: values are unchanged. 4096^2 relay
+// with a 1024-pixel pupil and stop: first pass 56 -> 29 us, last 53 -> 31, 828 -> 770 in all.
+struct RowLimits {
+    int first_in = -1, last_out = -1;
+    bool internal = false;                // maps and stores are the library's own (wfc.cu)
+};
+
+void limit_rows(int n, std::vector<Op>& ops, const RowLimits& lim) {
+    const int last = (int)ops.size() - 1;
+    for (int i = 0; i <= last; ++i) {
+        Op& op = ops[i];
+        if (!op.row) continue;
+        int r = op.mask_r;
+        if (r >= 0 && !lim.internal && (op.mask_map || op.mask_store)) r = -1;
+        if (i == 0 && !(op.row_flags & RF_INIT_ONE) && !lim.internal) r = -1;
+        const bool wanted = i == last && lim.last_out >= 0;
+        if (wanted && (r < 0 || lim.last_out < r)) r = lim.last_out;
+        if (i == 0 && lim.first_in >= 0 && (r < 0 || lim.first_in < r)) r = lim.first_in;
+        if (r < 0 || (i < last && ops[i + 1].lines != -9)) continue;   // the next pass reads every row
+        const int lo = std::max(0, n / 2 - r) / 256, hi = (std::min(n, n / 2 + r + 1) + 255) / 256;
+        if ((hi - lo) * 256 >= n) continue;
+        op.row_lo = lo * 256;
+        op.row_hi = hi * 256;
+        if (i == last && !wanted) op.row_flags |= RF_ZERO_REST;
+        if (i > 0 && ops[i - 1].lines == -9) { ops[i - 1].out_lo = lo; ops[i - 1].out_hi = hi; }
+        if (i < last) { ops[i + 1].in_lo = lo; ops[i + 1].in_hi = hi; }
+    }
 }
 
 // ev (optional, ops.size() + 1 events): recorded before the first pass and after each.
@@ -670,6 +713,8 @@ coro_status run_ops(coro_ctx ctx, int n, int batch, const std::vector<Op>& ops, 
             a.tw = op.variant == 5 ? tw_lin : tw;
             a.flags = op.row_flags;
             a.err = ctx->err;
+            a.row_lo = op.row_hi ? op.row_lo : 0;
+            a.row_hi = op.row_hi ? op.row_hi : n;
             a.elems = op.elems;
             pl.variant = op.variant;
             e = launch_row_pass<C>(n, a, pl);
@@ -682,6 +727,10 @@ coro_status run_ops(coro_ctx ctx, int n, int batch, const std::vector<Op>& ops, 
             a.tab_y = (const C*)op.tab_y;
             a.flags = op.col_flags;
             a.err = ctx->err;
+            a.in_lo = op.in_hi ? op.in_lo : 0;
+            a.in_hi = op.in_hi ? op.in_hi : n / 256;
+            a.out_lo = op.out_hi ? op.out_lo : 0;
+            a.out_hi = op.out_hi ? op.out_hi : n / 256;
             e = launch_col_pass<C>(n, op.lines, a, pl);
         }
         if (e != cudaSuccess) return cuda_fail(e, op.row ? "row pass" : "column pass");
@@ -1020,6 +1069,7 @@ struct FresnelPlan : coro_plan_s {
     std::vector<Op> ops_nat;         // the same passes, every one in place on the natural layout
     void* tbuf = nullptr;            // transposed plane of the alternating layout (owned)
     bool interleaved = false;        // ops run on interleaved row pairs (interleaved_ops)
+    RowLimits limits;
     DevBlocks db;
     std::vector<double> ps_final;
     std::vector<std::string> tune_log;
@@ -1131,6 +1181,8 @@ coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0,
     for (int p = 0; p < n_planes; ++p) {
         plan->plane_pitch[p] = ps;
         PassElems pe{};
+        int mask_r = -1;
+        bool mask_map = false, mask_store = false;
         auto push = [&](const DevElem& e) -> bool {
             if (pe.count >= kMaxPassElems - 3) {
                 set_error("plane %d: more than %d elements", p, kMaxPassElems - 3);
@@ -1145,7 +1197,19 @@ coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0,
         }
         for (const coro_element* el : planes[p].user) {
             DevElem e;
-            if ((st = compile_element(plan->db, el, dbl, n, batch, ps.data(), lam, &e)) != CORO_OK) return st;
+            if ((st = compile_element(plan->db, el, dbl, n, batch, ps.data(), lam, &e, plan->limits.internal)) != CORO_OK) return st;
+            if (el->kind == CORO_EL_APERTURE || (el->kind == CORO_EL_CIRCLE && !(el->flags & CORO_ELF_OPAQUE_INSIDE))) {
+                int r = 0;
+                for (int b = 0; b < batch; ++b) {
+                    const long long t = std::min<long long>(std::max<long long>(disk_threshold(el->radius, ps[b], false), 0), 4LL * n * n);
+                    int k = (int)std::sqrt((double)t) + 1;
+                    while ((long long)k * k > t) --k;
+                    r = std::max(r, k);
+                }
+                mask_r = mask_r < 0 ? r : std::min(mask_r, r);
+            }
+            mask_map = mask_map || (mask_r >= 0 && el->kind == CORO_EL_OPD_MAP);
+            mask_store = mask_store || el->kind == CORO_EL_CHECKPOINT || el->kind == CORO_EL_PHASE_GRAD;
             // after an angular-spectrum hop the row pass holds the field times (-1)^(x+y)
             // (the fftshift sign is carried into the next forward FFT); checkpoints undo it
             if ((e.kind == DK_STORE || e.kind == DK_PHASE_GRAD) && state == SPECTRUM) e.flags |= 1;
@@ -1159,6 +1223,9 @@ coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0,
         Op r;
         r.row = true;
         r.elems = pe;
+        r.mask_r = mask_r;
+        r.mask_map = mask_map;
+        r.mask_store = mask_store;
         if (state == SPECTRUM) r.row_flags |= RF_INV_FIRST;
         if (state == UNIFORM) r.row_flags |= RF_INIT_ONE;
         if (p + 1 < n_planes) {
@@ -1217,6 +1284,7 @@ void choose_layout(FresnelPlan* p) {
     }
     std::vector<Op> nat = p->ops_nat, il;
     if (!interleaved_ops(p->dtype, p->n, nat, &il)) return;
+    limit_rows(p->n, il, p->limits);
     if (autotune_enabled()) {
         coro_status st = CORO_OK;
         const size_t bytes = (size_t)p->batch * p->n * p->n * sizeof(float2);
@@ -1262,7 +1330,9 @@ std::unique_ptr<FresnelPlan> new_plan(coro_ctx ctx, int dtype, int n, int batch)
 
 }  // namespace
 
-extern "C" coro_status coro_fresnel_plan_create(coro_ctx ctx, const coro_fresnel_desc* d, coro_plan* out) {
+namespace {
+
+coro_status make_plan(coro_ctx ctx, const coro_fresnel_desc* d, const RowLimits& limits, coro_plan* out) {
     clear_error();
     if (!ctx || !d || !out) { set_error("coro_fresnel_plan_create: NULL argument"); return CORO_EINVAL; }
     *out = nullptr;
@@ -1283,6 +1353,7 @@ extern "C" coro_status coro_fresnel_plan_create(coro_ctx ctx, const coro_fresnel
     DeviceGuard g(ctx->device);
     auto plan = new_plan(ctx, d->dtype, d->n, d->batch);
     if (!plan) { set_error("out of host memory"); return CORO_ENOMEM; }
+    plan->limits = limits;
     std::vector<PlaneSpec> planes(d->n_planes);
     std::vector<HopSpec> hops(d->n_planes > 0 ? d->n_planes - 1 : 0);
     for (int i = 0; i < d->n_elements; ++i) planes[d->elements[i].plane].user.push_back(&d->elements[i]);
@@ -1293,6 +1364,28 @@ extern "C" coro_status coro_fresnel_plan_create(coro_ctx ctx, const coro_fresnel
     if ((st = build_passes(plan.get(), d->n, d->batch, d->pixelscale, d->wavelength, planes, hops, d->flags)) != CORO_OK)
         return st;
     return finish_plan(ctx, plan, out, "coro_fresnel_plan_create");
+}
+
+}  // namespace
+
+extern "C" coro_status coro_fresnel_plan_create(coro_ctx ctx, const coro_fresnel_desc* d, coro_plan* out) {
+    return make_plan(ctx, d, RowLimits{}, out);
+}
+
+coro_status coro::fresnel_plan_create_limited(coro_ctx ctx, const coro_fresnel_desc* d, int first_in, int last_out, coro_plan* out) {
+    RowLimits l;
+    l.first_in = first_in;
+    l.last_out = last_out;
+    l.internal = true;
+    return make_plan(ctx, d, l, out);
+}
+
+bool coro::fresnel_plan_rows(coro_plan plan, int pass, int* lo, int* hi) {
+    auto* p = static_cast<FresnelPlan*>(plan);
+    const Op& op = p->ops[pass];
+    *lo = op.row_hi ? op.row_lo : 0;
+    *hi = op.row_hi ? op.row_hi : p->n;
+    return op.row_hi != 0;
 }
 
 // ------------------------------------------------------------------------------ f2: pilot beam
@@ -1594,7 +1687,10 @@ extern "C" coro_status coro_fresnel_plan_copy_tuning(coro_plan dst, coro_plan sr
     d->ops = d->ops_nat;
     coro_status st = set_layout(d, 0);
     if (st == CORO_OK && s->tbuf) st = set_layout(d, 1);
-    if (st == CORO_OK && s->interleaved) d->interleaved = interleaved_ops(d->dtype, d->n, d->ops_nat, &d->ops) > 0;
+    if (st == CORO_OK && s->interleaved) {
+        d->interleaved = interleaved_ops(d->dtype, d->n, d->ops_nat, &d->ops) > 0;
+        limit_rows(d->n, d->ops, d->limits);
+    }
     return st;
 }
 

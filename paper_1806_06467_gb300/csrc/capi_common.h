@@ -137,6 +137,17 @@ coro_status lyot64_execute(coro_plan plan, const void* pupil, const double* peak
                            double* dh);
 
 
+// CORO_EL_OPD_MAP element flag of the library's own plans: the map's negative.
+constexpr int kElfMapNegate = 0x40000000;
+// A Fresnel plan of the library's own (maps finite where the field is, stores read only inside the
+// rows that run): first_in, last_out as in RowLimits (capi.cu), -1: none.
+coro_status fresnel_plan_create_limited(coro_ctx ctx, const coro_fresnel_desc* d, int first_in, int last_out, coro_plan* out);
+// Rows [*lo, *hi) of each item that (row) pass `pass` runs; false: all.
+bool fresnel_plan_rows(coro_plan plan, int pass, int* lo, int* hi);
+// coro_dm_correlate over rows [row_lo, row_hi) of w, the others taken as zeros (dm.cu).
+coro_status dm_correlate_rows(coro_ctx ctx, const float* w, int batch, int n, double pixelscale, int na, double pitch,
+                              double fwhm, double scale, int row_lo, int row_hi, float* grad);
+
 // Stream-ordered copy of a host array into a fresh device block (freed with free_async).
 void* upload_async(coro_ctx ctx, const void* host, size_t bytes, coro_status* st);
 void free_async(coro_ctx ctx, void* p);

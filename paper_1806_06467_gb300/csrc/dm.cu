@@ -21,6 +21,7 @@ struct DmGeom {
     int n, na;
     float dx, pitch, inv2s2;              // inv2s2 = 1 / (2 sigma^2)
     int half_win;                         // actuators on each side of the nearest one
+    int row_lo, row_hi;                   // transpose: rows of w that are read (the others count as zeros)
 };
 
 __device__ __forceinline__ float gauss(float d, float inv2s2) { return __expf(-d * d * inv2s2); }
@@ -53,8 +54,9 @@ __global__ void dm_correlate_kernel(const float* __restrict__ w, DmGeom g, float
     const float xa = ((float)q - c0) * g.pitch, ya = ((float)p - c0) * g.pitch;
     const float reach = (float)(g.half_win + 1) * g.pitch;
     const int x0 = max(0, (int)floorf((xa - reach) / g.dx) + g.n / 2), x1 = min(g.n - 1, (int)ceilf((xa + reach) / g.dx) + g.n / 2);
-    const int y0 = max(0, (int)floorf((ya - reach) / g.dx) + g.n / 2), y1 = min(g.n - 1, (int)ceilf((ya + reach) / g.dx) + g.n / 2);
-    const int wx = x1 - x0 + 1, wy = y1 - y0 + 1;
+    const int y0 = max(g.row_lo, (int)floorf((ya - reach) / g.dx) + g.n / 2);
+    const int y1 = min(g.row_hi - 1, (int)ceilf((ya + reach) / g.dx) + g.n / 2);
+    const int wx = x1 - x0 + 1, wy = max(0, y1 - y0 + 1);
     const float* wb = w + (size_t)b * g.n * g.n;
     double acc = 0.0;
     for (int i = threadIdx.x; i < wx * wy; i += blockDim.x) {
@@ -174,7 +176,7 @@ dm_correlate_u(const float* __restrict__ w, DmGeom g, int len, int span, const f
     const int xs0 = xs_tab[0];
     const int y = xs0 + r;
     float* ub = U + ((size_t)b * span + r) * g.na;
-    if (y < 0 || y >= g.n) {
+    if (y < g.row_lo || y >= g.row_hi) {
         for (int q = lane; q < g.na; q += 32) ub[q] = 0.f;
         return;
     }
@@ -283,6 +285,8 @@ coro_status geom(const char* fn, int n, int na, double pitch, double fwhm, doubl
     g->pitch = (float)pitch;
     g->inv2s2 = (float)(1.0 / (2.0 * sigma * sigma));
     g->half_win = (int)std::ceil(kWindowSigmas * sigma / pitch) + 1;
+    g->row_lo = 0;
+    g->row_hi = n;
     return CORO_OK;
 }
 
@@ -313,12 +317,19 @@ extern "C" coro_status coro_dm_opd(coro_ctx ctx, const float* heights, int batch
 
 extern "C" coro_status coro_dm_correlate(coro_ctx ctx, const float* w, int batch, int n, double pixelscale, int na,
                                          double pitch, double fwhm, double scale, float* grad) {
+    return coro::dm_correlate_rows(ctx, w, batch, n, pixelscale, na, pitch, fwhm, scale, 0, n, grad);
+}
+
+coro_status coro::dm_correlate_rows(coro_ctx ctx, const float* w, int batch, int n, double pixelscale, int na, double pitch,
+                                    double fwhm, double scale, int row_lo, int row_hi, float* grad) {
     coro::clear_error();
     if (!ctx || !w || !grad) { coro::set_error("coro_dm_correlate: NULL argument"); return CORO_EINVAL; }
     if (batch < 1 || batch > 65535) { coro::set_error("coro_dm_correlate: batch %d", batch); return CORO_ESIZE; }
     DmGeom g;
     coro_status st = geom("coro_dm_correlate", n, na, pitch, fwhm, pixelscale, &g);
     if (st != CORO_OK) return st;
+    g.row_lo = row_lo;
+    g.row_hi = row_hi;
     coro::DeviceGuard dg(ctx->device);
     int len = 0, span = 0;
     cudaError_t e = cudaSuccess;

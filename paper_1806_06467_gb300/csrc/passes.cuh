@@ -515,7 +515,8 @@ enum RowFlags : int {
     RF_FWD_AFTER = 2,     // forward row FFT after the elements
     RF_INIT_ONE = 4,      // do not read: the field starts as 1 + 0i
     RF_IN_IL = 8,         // packed-pair kernel only: rows 2m and 2m + 1 are read, or
-    RF_OUT_IL = 16        // written, sample by sample interleaved (see col_pass_pair_kernel)
+    RF_OUT_IL = 16,       // written, sample by sample interleaved (see col_pass_pair_kernel)
+    RF_ZERO_REST = 32     // packed-pair kernel only: rows outside [row_lo, row_hi) become zeros
 };
 
 template <typename C>
@@ -525,6 +526,9 @@ struct RowArgs {
     const C* tw;          // twiddles for N
     int flags;
     int* err;             // bounded-wait failure flag (persistent kernel)
+    // packed-pair kernel only: the rows of every item this pass transforms (even bounds, all by default);
+    // the others hold zeros that nobody reads (or writes, but for RF_ZERO_REST)
+    int row_lo, row_hi;
     PassElems elems;
 };
 
@@ -687,6 +691,9 @@ struct ColArgs {
     const C* tab_y;       // [batch][N]
     int flags;
     int* err;             // bounded-wait failure flag (persistent kernel)
+    // packed-pair kernel on interleaved rows only: 256-row boxes of the input that can hold non-zeros
+    // (the others are not read), and of the output that are wanted; all by default
+    int in_lo, in_hi, out_lo, out_hi;
 };
 
 template <int N, int L> struct ColCfg {
@@ -970,10 +977,11 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
         const int x = (g % GPI) * 2, y = (g / GPI) * N;
         float2* dst = stage + (k % S) * Cfg::GROUP;
         uint64_t* bar = &full[k % U];
-        tc::mbar_arrive_expect_tx(bar, BYTES);
+        const int q_lo = IL ? a.in_lo : 0, q_hi = IL ? a.in_hi : Cfg::BOXES;
+        tc::mbar_arrive_expect_tx(bar, (q_hi - q_lo) * 4096);      // 256 rows x 2 samples
 #pragma unroll 1
-        for (int q = 0; q < (IL ? N / 512 : Cfg::BOXES); ++q) {
-            if constexpr (IL) tc::tma_load_2d(dst + q * 1024, &map, bar, 2 * x, y / 2 + q * 256);
+        for (int q = q_lo; q < q_hi; ++q) {
+            if constexpr (IL) tc::tma_load_2d(dst + q * 512, &map, bar, 2 * x, y / 2 + q * 128);
             else tc::tma_load_2d(dst + q * 512, &map, bar, x, y + q * 256);
         }
     };
@@ -997,8 +1005,12 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
             const float2* src2 = stage + (k % S) * Cfg::GROUP;
 #pragma unroll
             for (int s = 0; s < 16; ++s) {
-                const float2 qa = src2[il_a + s * 2 * Cfg::TPL], qb = src2[il_b + s * 2 * Cfg::TPL];
-                v[s] = CP{pk::pack(qa.x, qb.x), pk::pack(qa.y, qb.y)};
+                const int q = s * Cfg::TPL / 256;                  // the box of rows t + s TPL
+                v[s] = CP{0ull, 0ull};
+                if (q >= a.in_lo && q < a.in_hi) {
+                    const float2 qa = src2[il_a + s * 2 * Cfg::TPL], qb = src2[il_b + s * 2 * Cfg::TPL];
+                    v[s] = CP{pk::pack(qa.x, qb.x), pk::pack(qa.y, qb.y)};
+                }
             }
         } else {
 #pragma unroll
@@ -1063,7 +1075,7 @@ col_pass_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __grid_con
                 tc::bulk_store(a.out + ((size_t)b * N + col) * N, region, BYTES);
             } else if constexpr (IL) {
 #pragma unroll 1
-                for (int q = 0; q < N / 512; ++q) tc::tma_store_2d(&map, region + q * 1024, 2 * col, b * (N / 2) + q * 256);
+                for (int q = a.out_lo; q < a.out_hi; ++q) tc::tma_store_2d(&map, region + q * 512, 2 * col, b * (N / 2) + q * 128);
             } else {
                 const int x = col, y = b * N;
 #pragma unroll 1
@@ -1416,9 +1428,12 @@ row_pass_pair_kernel(const __grid_constant__ RowArgs<float2> a, const __grid_con
     const SyncNamed sync{1 + u, Cfg::UT};
     const bool leader = t == 0;
     const bool load = !(a.flags & RF_INIT_ONE);
+    // pair g of the walk over the items' rows [row_lo, row_hi) -> pair of the whole field
+    const int band = (a.row_hi - a.row_lo) / 2;
+    auto pair_of = [&](int g) { return band == N / 2 ? g : g / band * (N / 2) + a.row_lo / 2 + g % band; };
 
     auto issue_load = [&](int k) {
-        const int g = blockIdx.x + k * gridDim.x;
+        const int g = pair_of(blockIdx.x + k * gridDim.x);
         uint64_t* bar = &full[k % U];
         float2* dst = stage + (k % S) * Cfg::GROUP;
         tc::mbar_arrive_expect_tx(bar, BYTES);
@@ -1439,10 +1454,19 @@ row_pass_pair_kernel(const __grid_constant__ RowArgs<float2> a, const __grid_con
             for (int k = 0; k < S && k < mine; ++k) issue_load(k);
     }
     __syncthreads();
+    if (a.flags & RF_ZERO_REST) {
+        const int rest = N / 2 - band, total = pairs / band * rest;
+        for (int z = blockIdx.x; z < total; z += gridDim.x) {
+            const int m = z % rest;
+            float4* o = reinterpret_cast<float4*>(a.out) +
+                        ((size_t)(z / rest) * (N / 2) + (m < a.row_lo / 2 ? m : m + band)) * (Cfg::GROUP / 2);
+            for (int i = threadIdx.x; i < Cfg::GROUP / 2; i += Cfg::THREADS) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
     bool ok = true;
     int j = 0;
     for (int k = u; k < mine; k += U, ++j) {
-        const int g = blockIdx.x + k * gridDim.x;       // row pair index over the batch
+        const int g = pair_of(blockIdx.x + k * gridDim.x);       // row pair index over the batch
         const int b = (2 * g) / N, ya = (2 * g) % N;
         CP v[16];
         if (load) {

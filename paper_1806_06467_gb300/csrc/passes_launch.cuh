@@ -138,7 +138,7 @@ cudaError_t col_launch_pair(const ColArgs<float2>& a, const PassLaunch& l) {
     if ((e = sm_count(&sms)) != cudaSuccess) return e;
     if ((a.in != a.out) != TOUT) return cudaErrorInvalidValue;
     CUtensorMap map;
-    e = IL ? tc_make_field_map(a.in, 2 * N, (long long)l.batch * N / 2, 4, &map, 256, true)
+    e = IL ? tc_make_field_map(a.in, 2 * N, (long long)l.batch * N / 2, 4, &map, 128, true)
            : tc_make_field_map(a.in, N, (long long)l.batch * N, 2, &map);
     if (e != cudaSuccess) return e;
     const int groups = l.batch * N / 2;
@@ -225,7 +225,8 @@ cudaError_t row_launch_pair(const RowArgs<float2>& a, const PassLaunch& l) {
         if (a.in == a.out || (a.flags & RF_INIT_ONE)) return cudaErrorInvalidValue;
         if ((e = tc_make_field_map(a.in, N, (long long)l.batch * N, 2, &map)) != cudaSuccess) return e;
     }
-    const int pairs = l.batch * N / 2;
+    const int pairs = l.batch * ((a.row_hi - a.row_lo) / 2);
+    if (pairs < 1 || (TIN && a.row_hi - a.row_lo != N)) return cudaErrorInvalidValue;
     const int grid = pairs < sms ? pairs : sms;
     row_pass_pair_kernel<N, U, S, TIN><<<grid, Cfg::THREADS, smem, l.stream>>>(a, map, pairs);
     return cudaGetLastError();

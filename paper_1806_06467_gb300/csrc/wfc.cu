@@ -67,7 +67,7 @@ struct WfcPlan : coro_plan_s {
     std::vector<Chunk> chunks;
     std::vector<void*> bufs;
     float2 *e1 = nullptr, *w = nullptr, *g = nullptr;
-    float *opd1 = nullptr, *opd1n = nullptr, *opd2 = nullptr, *opd2n = nullptr, *zero_h = nullptr;
+    float *opd1 = nullptr, *opd2 = nullptr, *zero_h = nullptr;
     float* part = nullptr;                      // [2][resident][n_act][n_act] per-wavelength dL/dh
     std::vector<double> peak;
     int kind() const override { return 3; }
@@ -107,9 +107,7 @@ coro_status dm_maps(WfcPlan* p, const float* heights) {
     const double dx = d.diam_m / d.npix;
     coro_status st;
     if ((st = coro_dm_opd(c, heights, 1, na, d.act_pitch_m, d.act_fwhm_m, nf, dx, 2.0, p->opd1)) != CORO_OK) return st;
-    if ((st = coro_dm_opd(c, heights, 1, na, d.act_pitch_m, d.act_fwhm_m, nf, dx, -2.0, p->opd1n)) != CORO_OK) return st;
-    if ((st = coro_dm_opd(c, heights + na * na, 1, na, d.act_pitch_m, d.act_fwhm_m, nf, dx, 2.0, p->opd2)) != CORO_OK) return st;
-    return coro_dm_opd(c, heights + na * na, 1, na, d.act_pitch_m, d.act_fwhm_m, nf, dx, -2.0, p->opd2n);
+    return coro_dm_opd(c, heights + na * na, 1, na, d.act_pitch_m, d.act_fwhm_m, nf, dx, 2.0, p->opd2);
 }
 
 coro_element checkpoint_elem(int plane, void* store) {
@@ -148,13 +146,15 @@ coro_status make_chunk(WfcPlan* p, Chunk& ch) {
     fd.n_elements = 4;
     fd.elements = fe;
     fd.flags = CORO_PLAN_INIT_UNIFORM;
-    if ((st = coro_fresnel_plan_create(p->ctx, &fd, &ch.fwd)) != CORO_OK) return st;
+    // the Lyot pupil is the centre window, all that is read of E3
+    if ((st = coro::fresnel_plan_create_limited(p->ctx, &fd, -1, d.npix / 2, &ch.fwd)) != CORO_OK) return st;
     // per-wavelength dL/dh density maps in w (E3 is no longer needed by then): DM2 first
     const size_t npx = (size_t)d.n_fresnel * d.n_fresnel;
     float* dphi2 = reinterpret_cast<float*>(p->w);
     float* dphi1 = dphi2 + (size_t)ch.nb * npx;
     coro_element ae[5]{};
-    ae[0] = opd_elem(p->opd2n);
+    ae[0] = opd_elem(p->opd2);                       // exp(-i phi2)
+    ae[0].flags = coro::kElfMapNegate;
     ae[0].plane = 1;
     ae[1].kind = CORO_EL_PHASE_GRAD;                 // (4 pi / lambda) 2 Im(G1 conj(E1))
     ae[1].plane = 1;
@@ -163,7 +163,8 @@ coro_status make_chunk(WfcPlan* p, Chunk& ch) {
     ae[1].store = dphi2;
     ae[2] = fe[0];                                   // A exp(-i phi1) G0 ...
     ae[2].plane = 2;
-    ae[3] = opd_elem(p->opd1n);
+    ae[3] = opd_elem(p->opd1);
+    ae[3].flags = coro::kElfMapNegate;
     ae[3].plane = 2;
     ae[4] = ae[1];                                   // ... (4 pi / lambda) 2 Im(A exp(-i phi1) G0)
     ae[4].plane = 2;
@@ -172,7 +173,8 @@ coro_status make_chunk(WfcPlan* p, Chunk& ch) {
     fd.n_elements = 5;
     fd.elements = ae;
     fd.flags = 0;
-    if ((st = coro_fresnel_plan_create(p->ctx, &fd, &ch.adj)) != CORO_OK) return st;
+    // G3 is zero outside the window, dL/dphi1 outside the aperture (and G0 is not read)
+    if ((st = coro::fresnel_plan_create_limited(p->ctx, &fd, d.npix / 2, d.npix / 2, &ch.adj)) != CORO_OK) return st;
     if ((st = coro_plan_set_graph(ch.fwd, 1)) != CORO_OK) return st;
     return coro_plan_set_graph(ch.adj, 1);
 }
@@ -236,10 +238,8 @@ extern "C" coro_status coro_wfc_plan_create(coro_ctx ctx, const coro_wfc_desc* d
     p->w = p->e1 ? (float2*)p->alloc(fbytes, &st) : nullptr;
     p->g = p->w ? (float2*)p->alloc(fbytes, &st) : nullptr;
     p->opd1 = p->g ? (float*)p->alloc(mbytes, &st) : nullptr;
-    p->opd1n = p->opd1 ? (float*)p->alloc(mbytes, &st) : nullptr;
-    p->opd2 = p->opd1n ? (float*)p->alloc(mbytes, &st) : nullptr;
-    p->opd2n = p->opd2 ? (float*)p->alloc(mbytes, &st) : nullptr;
-    p->zero_h = p->opd2n ? (float*)p->alloc((size_t)2 * d->n_act * d->n_act * sizeof(float), &st) : nullptr;
+    p->opd2 = p->opd1 ? (float*)p->alloc(mbytes, &st) : nullptr;
+    p->zero_h = p->opd2 ? (float*)p->alloc((size_t)2 * d->n_act * d->n_act * sizeof(float), &st) : nullptr;
     p->part = p->zero_h ? (float*)p->alloc((size_t)2 * R * d->n_act * d->n_act * sizeof(float), &st) : nullptr;
     if (!p->part) return st;
     cudaError_t e = cudaMemsetAsync(p->zero_h, 0, (size_t)2 * d->n_act * d->n_act * sizeof(float), ctx->stream);
@@ -312,15 +312,22 @@ extern "C" coro_status coro_wfc_plan_evaluate(coro_plan plan, const float* heigh
                                         dh.data() + ch.b0);
             continue;
         }
-        cudaError_t e = cudaMemsetAsync(p->g, 0, (size_t)nb * npx * sizeof(float2), c->stream);   // pad(): zero outside the window
+        // pad(): zero outside the window, in the rows that the adjoint's first pass reads
+        int lo = 0, hi = nf, g_lo = 0, g_hi = nf, launches = 0;
+        coro::fresnel_plan_rows(ch.adj, 0, &lo, &hi);
+        cudaError_t e = cudaMemset2DAsync(p->g + (size_t)lo * nf, npx * sizeof(float2), 0, (size_t)(hi - lo) * nf * sizeof(float2),
+                                          nb, c->stream);
         if (e != cudaSuccess) return coro::cuda_fail(e, "wfc: memset");
         st = coro_lyot_plan_gradient(ch.lyot, window(p, p->w), p->peak.data() + ch.b0, dh.data() + ch.b0,
                                      window(p, p->g), nf, (long long)nf * nf);
         // G3 -> G0 (in g), the row passes writing the per-wavelength dL/dh density maps into w
         if (st == CORO_OK) st = coro_fresnel_plan_execute(ch.adj, p->g, nullptr);
         const float* dphi2 = reinterpret_cast<const float*>(p->w);
+        if (st == CORO_OK) st = coro_plan_launch_count(ch.adj, &launches);
+        if (st == CORO_OK) coro::fresnel_plan_rows(ch.adj, launches - 1, &g_lo, &g_hi);
         if (st == CORO_OK)
-            st = coro_dm_correlate(c, dphi2 + (size_t)nb * npx, nb, nf, dx, na, d.act_pitch_m, d.act_fwhm_m, 1.0, p->part);
+            st = coro::dm_correlate_rows(c, dphi2 + (size_t)nb * npx, nb, nf, dx, na, d.act_pitch_m, d.act_fwhm_m, 1.0, g_lo, g_hi,
+                                         p->part);
         if (st == CORO_OK)
             st = coro_dm_correlate(c, dphi2, nb, nf, dx, na, d.act_pitch_m, d.act_fwhm_m, 1.0, p->part + (size_t)nb * per);
         if (st == CORO_OK) {

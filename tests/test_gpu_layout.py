@@ -212,6 +212,52 @@ def test_pass_flops(ctx):
     assert all(x == 2 * one for x in f[1:-1])
 
 
+@pytest.mark.parametrize("n", [1024, 2048, 4096])
+@pytest.mark.parametrize("r_first,r_mid,r_last", [(0.5, 0.13, 0.2), (0.02, 0.0, 0.49), (0.1, 0.3, 0.0)])
+def test_rows_left_out_behind_masks(ctx, n, r_first, r_mid, r_last):
+    """A uniform beam through an aperture, a stop between two hops, and a last stop (radii in units of
+    the grid: single rows, box edges, nearly all rows): transforming only the rows that the masks
+    leave gives bitwise the field of all rows, zeros where the last stop blocks, and the same for a
+    plan that takes the first one's kernels. A checkpoint behind a mask keeps every row."""
+    import os
+    lam, dx = np.array([500e-9, 640e-9]), 1.0 / n
+
+    def make(env, check):
+        els = [coro.element(coro.EL_APERTURE, plane=0, radius=r_first, obscuration=0.2, n_spiders=4, spider_width=3 * dx),
+               coro.element(coro.EL_CIRCLE, plane=1, radius=r_mid), coro.element(coro.EL_LENS, plane=2, focal_length=9.0),
+               coro.element(coro.EL_CIRCLE, plane=3, radius=r_last)]
+        if check is not None:
+            els.append(coro.element(coro.EL_CHECKPOINT, plane=1, store=check))
+        os.environ.update(env)
+        try:
+            return coro.FresnelPlan(ctx, n=n, batch=2, pixelscale=dx, wavelength=lam, distances=[1.5, -2.0, 3.0], elements=els,
+                                    init_uniform=True)
+        finally:
+            for k in env:
+                os.environ.pop(k)
+
+    natural = {"CORO_AUTOTUNE": "0", "CORO_LAYOUT": "0"}
+    fields = []
+    for env, check in ((natural, False), ({"CORO_AUTOTUNE": "0"}, False), ({"CORO_AUTOTUNE": "0"}, True)):
+        store = torch.full((2, n, n), float("nan"), dtype=torch.complex64, device="cuda") if check else None
+        plan = make(env, store)
+        x = torch.full((2, n, n), float("nan"), dtype=torch.complex64, device="cuda")     # not read
+        plan.execute(x)
+        fields.append(x)
+        if check:
+            assert bool(torch.isfinite(torch.view_as_real(store)).all())
+        elif len(fields) == 2:
+            other = make(natural, None)
+            other.copy_tuning(plan)
+            y = torch.full((2, n, n), float("nan"), dtype=torch.complex64, device="cuda")
+            other.execute(y)
+            assert torch.equal(x, y)
+            y.fill_(1.0)
+            plan.execute_range(y, 0, plan.launch_count)
+            assert torch.equal(x, y)
+    assert torch.equal(fields[0], fields[1]) and torch.equal(fields[0], fields[2])
+
+
 @pytest.mark.parametrize("n,batch", [(1024, 3), (2048, 2), (4096, 1)])
 def test_interleaved_row_pairs_match_natural_layout(ctx, n, batch):
     """A plan as created untuned (row pairs interleaved between passes), with a checkpoint, a direct
