@@ -7,6 +7,7 @@
 #include <complex>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdlib>
 #include <algorithm>
 #include <cstring>
@@ -237,19 +238,55 @@ const void* get_twiddles(coro_ctx ctx, int n, bool dbl, coro_status* st, bool li
     return p;
 }
 
+// A block of the context's arena for stream-ordered use on its stream, or NULL (too large, arena
+// full or absent, stream under capture). Blocks are handed out one after the other and all taken
+// back when the last of them is freed: a freed block is only reused by work that the stream
+// orders after its users, as with the stream-ordered allocator, which the arena stands in front of: that
+// one gives its memory back to the driver at every synchronisation, and a call that follows one then
+// waits some 200 us for it (a 256^2 hop alone: 251 us, with the arena 47).
+static void* arena_take(coro_ctx ctx, size_t bytes) {
+    constexpr size_t kArena = 2u << 20;
+    bytes = (bytes + 255) & ~(size_t)255;
+    if (bytes > kArena / 4) return nullptr;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
+    std::lock_guard<std::mutex> lock(ctx->arena_lock);
+    if (ctx->arena_off) return nullptr;
+    if (!ctx->arena) {
+        if (cudaMalloc(&ctx->arena, kArena) != cudaSuccess) {
+            ctx->arena = nullptr;
+            cudaGetLastError();
+            return nullptr;
+        }
+        ctx->arena_bytes = kArena;
+    }
+    if (ctx->arena_used + bytes > ctx->arena_bytes) return nullptr;
+    void* p = static_cast<char*>(ctx->arena) + ctx->arena_used;
+    ctx->arena_used += bytes;
+    ++ctx->arena_live;
+    return p;
+}
+
+static bool arena_give(coro_ctx ctx, void* p) {
+    std::lock_guard<std::mutex> lock(ctx->arena_lock);
+    if (!ctx->arena || p < ctx->arena || p >= static_cast<char*>(ctx->arena) + ctx->arena_bytes) return false;
+    if (--ctx->arena_live == 0) ctx->arena_used = 0;
+    return true;
+}
+
 void* upload_async(coro_ctx ctx, const void* host, size_t bytes, coro_status* st) {
-    void* p = nullptr;
-    cudaError_t e = cudaMallocAsync(&p, bytes, ctx->stream);
+    void* p = arena_take(ctx, bytes);
+    cudaError_t e = p ? cudaSuccess : cudaMallocAsync(&p, bytes, ctx->stream);
     if (e != cudaSuccess) { *st = cuda_fail(e, "cudaMallocAsync"); return nullptr; }
     if (host) {
         e = cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, ctx->stream);
-        if (e != cudaSuccess) { cudaFreeAsync(p, ctx->stream); *st = cuda_fail(e, "cudaMemcpyAsync"); return nullptr; }
+        if (e != cudaSuccess) { free_async(ctx, p); *st = cuda_fail(e, "cudaMemcpyAsync"); return nullptr; }
     }
     return p;
 }
 
 void free_async(coro_ctx ctx, void* p) {
-    if (p) cudaFreeAsync(p, ctx->stream);
+    if (p && !arena_give(ctx, p)) cudaFreeAsync(p, ctx->stream);
 }
 
 void* ctx_work(coro_ctx ctx, size_t bytes, coro_status* st) {
@@ -304,6 +341,7 @@ extern "C" coro_status coro_ctx_destroy(coro_ctx ctx) {
         for (auto& kv : ctx->tw64) cudaFree(kv.second);
         if (ctx->work) cudaFree(ctx->work);
         if (ctx->err) cudaFree(ctx->err);
+        if (ctx->arena) cudaFree(ctx->arena);
     }
     delete ctx;
     return CORO_OK;
@@ -313,6 +351,8 @@ extern "C" coro_status coro_ctx_set_stream(coro_ctx ctx, void* stream) {
     clear_error();
     if (!ctx) { set_error("coro_ctx_set_stream: ctx is NULL"); return CORO_EINVAL; }
     ctx->stream = (cudaStream_t)stream;
+    std::lock_guard<std::mutex> lock(ctx->arena_lock);
+    ctx->arena_off = true;               // its order is that of the context's first stream
     return CORO_OK;
 }
 
@@ -1771,14 +1811,52 @@ extern "C" coro_status coro_plan_destroy(coro_plan plan) {
 
 namespace {
 
+// (re^2 + im^2) / norm, rounded once: complex64 samples in two-float arithmetic (squares and their sum
+// exact to 2^-46, the product with 1 / norm = sh + sl alike), because FP64 runs at 1/64 of the FP32 rate
+// here: 2048^2 (50 MB) took 51 us in FP64, 12 us like this. Sums and results outside [1e-30, 1e30],
+// where a part would under- or overflow, take FP64.
+// (a call: predicated, its instructions would occupy the FP64 pipe for every sample)
+__device__ __noinline__ float intensity_fp64(float2 v, double s) { return (float)(((double)v.x * v.x + (double)v.y * v.y) * s); }
+
+__device__ __forceinline__ float intensity_of(float2 v, double s, float sh, float sl) {
+    const float p = v.x * v.x, q = v.y * v.y, h = p + q;
+    if (v.x == 0.f && v.y == 0.f) return 0.f;            // outside a stop; s is finite
+    const float r = h * sh;
+    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f)) return intensity_fp64(v, s);
+    const float ep = fmaf(v.x, v.x, -p), eq = fmaf(v.y, v.y, -q), bb = h - p;
+    const float l = ((p - (h - bb)) + (q - bb)) + (ep + eq);
+    return r + (fmaf(h, sh, -r) + (h * sl + l * sh));
+}
+
+// grid.y: items. Two samples per thread and step where they sit on a 16-byte boundary.
 template <typename C>
-__global__ void intensity_kernel(const C* __restrict__ e, float* __restrict__ out, size_t per_item,
-                                 int batch, const double* __restrict__ inv_norm) {
-    const size_t total = per_item * batch;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const C v = e[i];
-        const double s = inv_norm[i / per_item];
-        out[i] = (float)(((double)v.x * v.x + (double)v.y * v.y) * s);
+__global__ void __launch_bounds__(256) intensity_kernel(const C* __restrict__ e, float* __restrict__ out, size_t per_item,
+                                                        const double* __restrict__ inv_norm) {
+    const double s = inv_norm[blockIdx.y];
+    e += blockIdx.y * per_item;
+    out += blockIdx.y * per_item;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    if constexpr (std::is_same<C, float2>::value) {
+        const float sh = (float)s, sl = (float)(s - (double)sh);
+        const bool plain = sh > 1e-30f && sh < 1e30f;     // 1 / norm held as two floats
+        size_t from = 0;
+        if (plain && !((uintptr_t)e & 15) && !((uintptr_t)out & 7)) {
+            for (size_t i = first; i < per_item / 2; i += step) {
+                const float4 v = reinterpret_cast<const float4*>(e)[i];
+                reinterpret_cast<float2*>(out)[i] = make_float2(intensity_of(make_float2(v.x, v.y), s, sh, sl),
+                                                                intensity_of(make_float2(v.z, v.w), s, sh, sl));
+            }
+            from = per_item & ~(size_t)1;
+        }
+        for (size_t i = from + first; i < per_item; i += step) {
+            const C v = e[i];
+            out[i] = plain ? intensity_of(v, s, sh, sl) : intensity_fp64(v, s);
+        }
+    } else {
+        for (size_t i = first; i < per_item; i += step) {
+            const C v = e[i];
+            out[i] = (float)((v.x * v.x + v.y * v.y) * s);
+        }
     }
 }
 
@@ -1825,9 +1903,10 @@ extern "C" coro_status coro_intensity(coro_ctx ctx, const coro_wavefront* wf, co
     void* inv_d = upload_async(ctx, inv.data(), inv.size() * sizeof(double), &st);
     if (!inv_d) return st;
     const size_t per = (size_t)wf->n * wf->n;
-    const int blocks = (int)std::min<size_t>((per * wf->batch + 255) / 256, 152 * 8);
-    if (wf->dtype == CORO_C64) intensity_kernel<float2><<<blocks, 256, 0, ctx->stream>>>((const float2*)wf->data, out, per, wf->batch, (const double*)inv_d);
-    else intensity_kernel<double2><<<blocks, 256, 0, ctx->stream>>>((const double2*)wf->data, out, per, wf->batch, (const double*)inv_d);
+    const int most = std::max(1, 152 * 8 / wf->batch);
+    const dim3 blocks((unsigned)std::min<size_t>((per / 2 + 255) / 256 + 1, most), wf->batch);
+    if (wf->dtype == CORO_C64) intensity_kernel<float2><<<blocks, 256, 0, ctx->stream>>>((const float2*)wf->data, out, per, (const double*)inv_d);
+    else intensity_kernel<double2><<<blocks, 256, 0, ctx->stream>>>((const double2*)wf->data, out, per, (const double*)inv_d);
     cudaError_t e = cudaGetLastError();
     free_async(ctx, inv_d);
     return e == cudaSuccess ? CORO_OK : cuda_fail(e, "intensity_kernel");

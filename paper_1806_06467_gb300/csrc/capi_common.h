@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -18,6 +19,12 @@ struct coro_ctx_s {
     void* work = nullptr;        // MFT work buffer (grown on demand)
     size_t work_bytes = 0;
     int* err = nullptr;          // device flag set by kernels whose bounded waits expired
+    // small stream-ordered blocks (upload_async): one device allocation, made on first use
+    std::mutex arena_lock;
+    void* arena = nullptr;
+    size_t arena_bytes = 0, arena_used = 0;
+    int arena_live = 0;
+    bool arena_off = false;      // after coro_ctx_set_stream
 };
 
 // Replay of a plan's launch sequence as one CUDA graph. The graph is captured on a private

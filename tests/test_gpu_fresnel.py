@@ -556,3 +556,28 @@ def test_intensity_and_darkhole(ctx):
     for b in range(3):
         ref = coronagraph.dark_hole_sum(np.abs(f32[b]) ** 2 / norm[b], du, 6.0, 20.0)
         assert abs(s[b] - ref) < 1e-12 * ref
+
+
+@pytest.mark.parametrize("n,batch", [(32, 3), (36, 1), (150, 2)])
+def test_intensity_rounds_once_over_the_whole_range(ctx, n, batch):
+    """Detector intensity of complex64 fields against FP64 rounded once: ordinary samples (aligned or not),
+    zeros, and squares that under- or overflow FP32 while the normalised value does not, item by item."""
+    g = np.random.default_rng(n)
+    f = (g.standard_normal((batch, n, n)) + 1j * g.standard_normal((batch, n, n))) * 10.0 ** g.uniform(-18, 18, (batch, n, n))
+    f[:, 0, :9] = 0.0
+    f[:, 1, 0] = complex("nan")
+    f[:, 1, 1] = complex("inf")
+    f = f.astype(np.complex64)
+    x = torch.from_numpy(f).cuda()
+    for norm in (np.full(batch, 1.0), 10.0 ** g.uniform(-12, 12, batch), np.full(batch, 1e-35)):
+        with np.errstate(all="ignore"):
+            ref = (f.real.astype(np.float64) ** 2 + f.imag.astype(np.float64) ** 2) * (1.0 / norm)[:, None, None]
+            ref32 = ref.astype(np.float32)
+        got = coro.intensity(ctx, x, norm).cpu().numpy()
+        plain = torch.empty(batch * n * n + 1, dtype=torch.float32, device="cuda")[1:]        # not on 8 bytes
+        coro.intensity(ctx, x, norm, out=plain)
+        assert np.array_equal(plain.cpu().numpy().reshape(got.shape), got, equal_nan=True)
+        fin = np.isfinite(ref32) & (ref32 >= np.finfo(np.float32).tiny)
+        assert np.all(np.abs(got[fin] - ref[fin]) <= 0.5001 * np.spacing(ref32[fin]))          # half a unit
+        assert np.array_equal(got[~np.isfinite(ref32)], ref32[~np.isfinite(ref32)], equal_nan=True)
+        assert np.all(got[ref == 0.0] == 0.0)
