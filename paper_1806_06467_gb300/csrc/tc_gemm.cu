@@ -233,10 +233,7 @@ tc_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ 
                     const int ky = n - it.N / 2;
                     const int r2 = kx * kx + ky * ky;
                     const bool keep = r2 >= it.mask_lo && r2 <= it.mask_hi;
-                    if constexpr (EPI == TC_EPI_C64T) {
-                        float2* d = reinterpret_cast<float2*>(a.dst) + b * a.dst_bstride + (size_t)n * a.dst_ld + m;
-                        *d = make_float2(re, im);
-                    } else if constexpr (EPI == TC_EPI_SPLITT) {
+                    if constexpr (EPI == TC_EPI_SPLITT) {
                         if (!keep) { re = 0.f; im = 0.f; }
                         const size_t plane = (size_t)a.dst_rows * a.dst_ld;
                         store_split<BF16>(a.dst, plane, b * a.dst_bstride + (size_t)n * a.dst_ld + m, re, im);
@@ -296,15 +293,14 @@ __global__ void split_kernel(const float2* __restrict__ src, long long sb, int s
 // fractional cycle, then rounded to FP32 and split. plane_rows = rows of the operand planes
 // (>= rows), item = first item written (grid z offsets from it).
 template <bool BF16>
-__global__ void basis_kernel(const double* __restrict__ c, double c_one, int sign, void* dst, int rows, int cols,
-                             int ld, int plane_rows, int item) {
+__global__ void basis_kernel(double c, int sign, void* dst, int rows, int cols, int ld, int plane_rows, int item) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y, b = blockIdx.z + item;
+    const int r = blockIdx.y;
     if (k >= ld) return;
     float re = 0.f, im = 0.f;
     if (k < cols) {
         const long long rr = (long long)r - rows / 2, kk = (long long)k - cols / 2;
-        double cyc = (double)(rr * kk) * (c ? c[b] : c_one);
+        double cyc = (double)(rr * kk) * c;
         cyc -= rint(cyc);
         double s, co;
         sincospi(2.0 * cyc, &s, &co);
@@ -312,7 +308,7 @@ __global__ void basis_kernel(const double* __restrict__ c, double c_one, int sig
         im = (float)(sign < 0 ? -s : s);
     }
     const size_t plane = (size_t)plane_rows * ld;
-    store_split<BF16>(dst, plane, (size_t)b * 4 * plane + (size_t)r * ld + k, re, im);
+    store_split<BF16>(dst, plane, (size_t)item * 4 * plane + (size_t)r * ld + k, re, im);
 }
 
 template <bool BF16>
@@ -422,14 +418,12 @@ cudaError_t tc_launch(bool bf16, int epi, const CUtensorMap& mx, const CUtensorM
     (void)max_k;
     if (bf16) {
         switch (epi) {
-            case TC_EPI_C64T: return launch_t<true, TC_EPI_C64T>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_SPLITT: return launch_t<true, TC_EPI_SPLITT>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_BABINET: return launch_t<true, TC_EPI_BABINET>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_INTENSITY: return launch_t<true, TC_EPI_INTENSITY>(mx, mw, max_m, max_n, batch, args, stream);
         }
     } else {
         switch (epi) {
-            case TC_EPI_C64T: return launch_t<false, TC_EPI_C64T>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_SPLITT: return launch_t<false, TC_EPI_SPLITT>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_BABINET: return launch_t<false, TC_EPI_BABINET>(mx, mw, max_m, max_n, batch, args, stream);
             case TC_EPI_INTENSITY: return launch_t<false, TC_EPI_INTENSITY>(mx, mw, max_m, max_n, batch, args, stream);
@@ -446,13 +440,6 @@ cudaError_t tc_split(bool bf16, const float2* src, long long src_bstride, int sr
     return cudaGetLastError();
 }
 
-cudaError_t tc_basis(bool bf16, const double* c, int sign, const TcOperand& dst, cudaStream_t stream) {
-    dim3 grid((dst.ld + 127) / 128, dst.rows, dst.batch);
-    if (bf16) basis_kernel<true><<<grid, 128, 0, stream>>>(c, 0.0, sign, dst.base, dst.rows, dst.cols, dst.ld, dst.rows, 0);
-    else basis_kernel<false><<<grid, 128, 0, stream>>>(c, 0.0, sign, dst.base, dst.rows, dst.cols, dst.ld, dst.rows, 0);
-    return cudaGetLastError();
-}
-
 cudaError_t tc_merge(bool bf16, const TcOperand& src, float2* dst, long long dst_bstride, int dst_ld,
                      cudaStream_t stream) {
     dim3 grid((src.cols + 127) / 128, src.rows, src.batch);
@@ -465,8 +452,8 @@ cudaError_t tc_basis_one(bool bf16, double c, int sign, const TcOperand& dst, in
                          int cols_valid, cudaStream_t stream) {
     if (rows_valid > dst.rows || cols_valid > dst.ld || item < 0 || item >= dst.batch) return cudaErrorInvalidValue;
     dim3 grid((dst.ld + 127) / 128, rows_valid, 1);
-    if (bf16) basis_kernel<true><<<grid, 128, 0, stream>>>(nullptr, c, sign, dst.base, rows_valid, cols_valid, dst.ld, dst.rows, item);
-    else basis_kernel<false><<<grid, 128, 0, stream>>>(nullptr, c, sign, dst.base, rows_valid, cols_valid, dst.ld, dst.rows, item);
+    if (bf16) basis_kernel<true><<<grid, 128, 0, stream>>>(c, sign, dst.base, rows_valid, cols_valid, dst.ld, dst.rows, item);
+    else basis_kernel<false><<<grid, 128, 0, stream>>>(c, sign, dst.base, rows_valid, cols_valid, dst.ld, dst.rows, item);
     return cudaGetLastError();
 }
 

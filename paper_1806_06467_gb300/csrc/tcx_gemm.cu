@@ -347,17 +347,6 @@ tcx_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__
             }
             // both warps have read the pair's maxima before either writes the next tile's
             asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-        } else if constexpr (EPI == TC_EPI_C64T) {
-            if (ok && m < it.M) {
-#pragma unroll
-                for (int j = 0; j < EPI_COLS; ++j) {
-                    const int n = n0 + cg * EPI_COLS + j;
-                    if (n < it.N) {
-                        float2* d = reinterpret_cast<float2*>(a.dst) + b * a.dst_bstride + (size_t)n * a.dst_ld + m;
-                        *d = make_float2(hr[j] + lr[j], hi_[j] + li[j]);
-                    }
-                }
-            }
         } else {
             // intensity |Y|^2 / peak in two-float; dark-hole sum and running peak in FP64
             const float ph = (float)it.inv_peak64, pl = (float)(it.inv_peak64 - (double)ph);
@@ -523,7 +512,6 @@ template <int BN>
 cudaError_t launch_bn(int epi, const CUtensorMap& mx, const CUtensorMap& mw, int max_m, int max_n, int batch,
                       const TcArgs& args, cudaStream_t stream) {
     switch (epi) {
-        case TC_EPI_C64T: return launch_t<BN, TC_EPI_C64T>(mx, mw, max_m, max_n, batch, args, stream);
         case TC_EPI_SPLITT: return launch_t<BN, TC_EPI_SPLITT>(mx, mw, max_m, max_n, batch, args, stream);
         case TC_EPI_BABINET: return launch_t<BN, TC_EPI_BABINET>(mx, mw, max_m, max_n, batch, args, stream);
         case TC_EPI_INTENSITY: return launch_t<BN, TC_EPI_INTENSITY>(mx, mw, max_m, max_n, batch, args, stream);
