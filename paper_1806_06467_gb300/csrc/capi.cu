@@ -686,37 +686,40 @@ int interleaved_ops(int dtype, int n, std::vector<Op>& nat, std::vector<Op>* out
     return found;
 }
 
-// Rows that cannot matter are left out of interleaved passes: behind a mask (an aperture or stop) only
+// Rows that cannot matter are left out of interleaved passes and of the mixed-radix packed-pair ones: behind a mask (an aperture or stop) only
 // the rows it leaves are transformed, written before it by the column pass and read after it by the
-// next one, in boxes of 256 rows; a plan's last row pass fills its other rows with zeros. first_in: rows
+// next one, in boxes of 256 rows (mixed radix: 200 or 2 x 205); a plan's last row pass fills its other rows with zeros. first_in: rows
 // n/2 +- first_in are all the input's non-zeros (-1: unknown); last_out: only rows n/2 +- last_out of the
 // result are wanted (-1: all; the others are then left as they are). The first plane's mask counts
 // where the plan makes the field itself (INIT_ONE), so that what a caller's field holds under the mask
 // reaches the passes as before. Skipped are products with zeros: values are unchanged. 4096^2 relay
-// with a 1024-pixel pupil and stop: first pass 56 -> 29 us, last 53 -> 31, 828 -> 770 in all.
+// with a 1024-pixel pupil and stop: first pass 56 -> 29 us, last 53 -> 31, 828 -> 770 in all; 2800^2
+// with 700 pixels 689 -> 630.
 struct RowLimits {
     int first_in = -1, last_out = -1;
     bool internal = false;                // maps and stores are the library's own (wfc.cu)
 };
 
 void limit_rows(int n, std::vector<Op>& ops, const RowLimits& lim) {
-    const int last = (int)ops.size() - 1;
+    const int last = (int)ops.size() - 1, box = col_box_rows(n), step = box % 2 ? 2 : 1;   // even bounds
+    if (!box) return;
     for (int i = 0; i <= last; ++i) {
         Op& op = ops[i];
-        if (!op.row) continue;
+        if (!op.row || !row_takes_band(n, op.variant)) continue;
         int r = op.mask_r;
         if (r >= 0 && !lim.internal && (op.mask_map || op.mask_store)) r = -1;
         if (i == 0 && !(op.row_flags & RF_INIT_ONE) && !lim.internal) r = -1;
         const bool wanted = i == last && lim.last_out >= 0;
         if (wanted && (r < 0 || lim.last_out < r)) r = lim.last_out;
         if (i == 0 && lim.first_in >= 0 && (r < 0 || lim.first_in < r)) r = lim.first_in;
-        if (r < 0 || (i < last && ops[i + 1].lines != -9)) continue;   // the next pass reads every row
-        const int lo = std::max(0, n / 2 - r) / 256, hi = (std::min(n, n / 2 + r + 1) + 255) / 256;
-        if ((hi - lo) * 256 >= n) continue;
-        op.row_lo = lo * 256;
-        op.row_hi = hi * 256;
+        if (r < 0 || (i < last && (ops[i + 1].row || !col_takes_band(n, ops[i + 1].lines)))) continue;   // the next pass reads every row
+        const int unit = box * step;
+        const int lo = std::max(0, n / 2 - r) / unit * step, hi = (std::min(n, n / 2 + r + 1) + unit - 1) / unit * step;
+        if ((hi - lo) * box >= n) continue;
+        op.row_lo = lo * box;
+        op.row_hi = hi * box;
         if (i == last && !wanted) op.row_flags |= RF_ZERO_REST;
-        if (i > 0 && ops[i - 1].lines == -9) { ops[i - 1].out_lo = lo; ops[i - 1].out_hi = hi; }
+        if (i > 0 && !ops[i - 1].row && col_takes_band(n, ops[i - 1].lines)) { ops[i - 1].out_lo = lo; ops[i - 1].out_hi = hi; }
         if (i < last) { ops[i + 1].in_lo = lo; ops[i + 1].in_hi = hi; }
     }
 }
@@ -741,6 +744,7 @@ coro_status run_ops(coro_ctx ctx, int n, int batch, const std::vector<Op>& ops, 
         const cudaError_t e0 = record_timing_event(ev[0], ctx->stream);
         if (e0 != cudaSuccess) return cuda_fail(e0, "cudaEventRecord");
     }
+    const int boxes = col_box_rows(n) ? n / col_box_rows(n) : 0;
     int i = 0;
     for (const Op& op : ops) {
         cudaError_t e;
@@ -768,9 +772,9 @@ coro_status run_ops(coro_ctx ctx, int n, int batch, const std::vector<Op>& ops, 
             a.flags = op.col_flags;
             a.err = ctx->err;
             a.in_lo = op.in_hi ? op.in_lo : 0;
-            a.in_hi = op.in_hi ? op.in_hi : n / 256;
+            a.in_hi = op.in_hi ? op.in_hi : boxes;
             a.out_lo = op.out_hi ? op.out_lo : 0;
-            a.out_hi = op.out_hi ? op.out_hi : n / 256;
+            a.out_hi = op.out_hi ? op.out_hi : boxes;
             e = launch_col_pass<C>(n, op.lines, a, pl);
         }
         if (e != cudaSuccess) return cuda_fail(e, op.row ? "row pass" : "column pass");
@@ -1109,6 +1113,7 @@ struct FresnelPlan : coro_plan_s {
     std::vector<Op> ops_nat;         // the same passes, every one in place on the natural layout
     void* tbuf = nullptr;            // transposed plane of the alternating layout (owned)
     bool interleaved = false;        // ops run on interleaved row pairs (interleaved_ops)
+    bool limited = false;            // ops leave rows out on the natural layout (mixed radix)
     RowLimits limits;
     DevBlocks db;
     std::vector<double> ps_final;
@@ -1174,7 +1179,7 @@ coro_status set_layout(FresnelPlan* p, int transposed) {
             p->tbuf = nullptr;
         }
     }
-    p->interleaved = false;
+    p->interleaved = p->limited = false;
     p->graph.reset();                                   // a captured graph holds the old kernels
     return CORO_OK;
 }
@@ -1323,7 +1328,12 @@ void choose_layout(FresnelPlan* p) {
         return;
     }
     std::vector<Op> nat = p->ops_nat, il;
-    if (!interleaved_ops(p->dtype, p->n, nat, &il)) return;
+    if (!interleaved_ops(p->dtype, p->n, nat, &il)) {
+        if (p->dtype != CORO_C64 || !(p->n & (p->n - 1))) return;
+        limit_rows(p->n, p->ops, p->limits);
+        p->limited = true;
+        return;
+    }
     limit_rows(p->n, il, p->limits);
     if (autotune_enabled()) {
         coro_status st = CORO_OK;
@@ -1727,7 +1737,8 @@ extern "C" coro_status coro_fresnel_plan_copy_tuning(coro_plan dst, coro_plan sr
     d->ops = d->ops_nat;
     coro_status st = set_layout(d, 0);
     if (st == CORO_OK && s->tbuf) st = set_layout(d, 1);
-    if (st == CORO_OK && s->interleaved) {
+    if (st == CORO_OK && (s->interleaved || s->limited)) {
+        d->limited = s->limited;
         d->interleaved = interleaved_ops(d->dtype, d->n, d->ops_nat, &d->ops) > 0;
         limit_rows(d->n, d->ops, d->limits);
     }

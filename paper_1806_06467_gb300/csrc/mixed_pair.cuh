@@ -348,8 +348,13 @@ row_pass_mixed_pair_kernel(const __grid_constant__ RowArgs<float2> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CP* buf = reinterpret_cast<CP*>(smem_raw);
     constexpr int S = (N + T - 1) / T;
-    const int ya = 2 * blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    // blocks cover the rows [row_lo, row_hi), or every row where the others become zeros
+    const int ya = 2 * blockIdx.x + (a.flags & RF_ZERO_REST ? 0 : a.row_lo), b = blockIdx.y, tid = threadIdx.x;
     const size_t ra = ((size_t)b * N + ya) * N, rb = ra + N;
+    if (ya < a.row_lo || ya >= a.row_hi) {
+        for (int x = tid; x < 2 * N; x += T) a.out[ra + x] = make_float2(0.f, 0.f);
+        return;
+    }
     // the two rows arrive by two bulk copies into the line buffer (dense, row A then row B),
     // then move through registers into the padded pair layout
     const bool bulk = !(a.flags & RF_INIT_ONE) && ((uintptr_t)a.in & 15) == 0;
@@ -472,6 +477,8 @@ col_pass_mixed_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __gr
     // TMA wants the staging boxes on 128-byte boundaries: a block whose shared memory were placed
     // otherwise would move its strip with plain loads and stores instead (same results)
     const bool tma = BR > 0 && (tc::smem_u32(stage) & 127u) == 0;
+    // rows that are read; the others are zeros (limit_rows)
+    const int in_lo = BR > 0 ? a.in_lo * BR : 0, in_hi = BR > 0 ? a.in_hi * BR : N;
     if (tma) {
         if (tid == 0) {
             tc::mbar_init(bar, 1);
@@ -480,9 +487,9 @@ col_pass_mixed_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __gr
         }
         __syncthreads();
         if (tid == 0) {
-            tc::mbar_arrive_expect_tx(bar, (uint32_t)(N * sizeof(CP)));
+            tc::mbar_arrive_expect_tx(bar, (uint32_t)((in_hi - in_lo) * sizeof(CP)));
 #pragma unroll 1
-            for (int q = 0; q < N / BR; ++q) tc::tma_load_2d(stage + q * BRP, &mi, bar, col, b * N + q * BR);
+            for (int q = a.in_lo; q < a.in_hi; ++q) tc::tma_load_2d(stage + q * BRP, &mi, bar, col, b * N + q * BR);
         }
         tc::mbar_wait(bar, 0, a.err, 16);
     }
@@ -492,7 +499,8 @@ col_pass_mixed_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __gr
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             const int y = tid + s * T;
-            if (S * T == N || y < N) q[s] = tma ? stage[srow(y)] : src[(size_t)y * ROW4];
+            if (y >= in_lo && y < in_hi) q[s] = tma ? stage[srow(y)] : src[(size_t)y * ROW4];
+            else q[s] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (tma) __syncthreads();                    // every staged row read before the rearrangement
 #pragma unroll
@@ -547,7 +555,7 @@ col_pass_mixed_pair_kernel(const __grid_constant__ ColArgs<float2> a, const __gr
         __syncthreads();
         if (tid == 0) {
 #pragma unroll 1
-            for (int q = 0; q < N / BR; ++q) tc::tma_store_2d(&mo, stage + q * BRP, col, b * N + q * BR);
+            for (int q = a.out_lo; q < a.out_hi; ++q) tc::tma_store_2d(&mo, stage + q * BRP, col, b * N + q * BR);
             tc::bulk_commit();
             tc::bulk_wait_read<0>();         // staging read out; the writes finish with the grid
         }
@@ -566,7 +574,9 @@ cudaError_t row_launch_mixed_pair_n(const RowArgs<float2>& a, const PassLaunch& 
     static unsigned done = 0;
     cudaError_t e = ensure_smem(row_pass_mixed_pair_kernel<N, T>, smem, done);
     if (e != cudaSuccess) return e;
-    row_pass_mixed_pair_kernel<N, T><<<dim3(N / 2, l.batch), T, smem, l.stream>>>(a);
+    const int rows = a.flags & RF_ZERO_REST ? N : a.row_hi - a.row_lo;
+    if (a.row_lo < 0 || a.row_hi > N || a.row_hi <= a.row_lo || a.row_lo % 2 || a.row_hi % 2) return cudaErrorInvalidValue;
+    row_pass_mixed_pair_kernel<N, T><<<dim3(rows / 2, l.batch), T, smem, l.stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -576,6 +586,8 @@ cudaError_t col_launch_mixed_pair_n(const ColArgs<float2>& a, const PassLaunch& 
     constexpr int T = mpair::pair_threads(N);
     constexpr int BR = mpair::pair_tma_rows(N);
     if (((uintptr_t)a.in & 15) || ((uintptr_t)a.out & 15)) return cudaErrorInvalidValue;
+    if (BR > 0 && (a.in_lo < 0 || a.in_hi * BR > N || a.in_hi <= a.in_lo || a.out_lo < 0 || a.out_hi * BR > N ||
+                   a.out_hi <= a.out_lo)) return cudaErrorInvalidValue;
     const size_t smem = mpair::pair_col_smem(N);
     static unsigned done = 0;
     cudaError_t e = ensure_smem(col_pass_mixed_pair_kernel<N, T, BR>, smem, done);

@@ -516,7 +516,7 @@ enum RowFlags : int {
     RF_INIT_ONE = 4,      // do not read: the field starts as 1 + 0i
     RF_IN_IL = 8,         // packed-pair kernel only: rows 2m and 2m + 1 are read, or
     RF_OUT_IL = 16,       // written, sample by sample interleaved (see col_pass_pair_kernel)
-    RF_ZERO_REST = 32     // packed-pair kernel only: rows outside [row_lo, row_hi) become zeros
+    RF_ZERO_REST = 32     // packed-pair kernels only: rows outside [row_lo, row_hi) become zeros
 };
 
 template <typename C>
@@ -526,7 +526,7 @@ struct RowArgs {
     const C* tw;          // twiddles for N
     int flags;
     int* err;             // bounded-wait failure flag (persistent kernel)
-    // packed-pair kernel only: the rows of every item this pass transforms (even bounds, all by default);
+    // packed-pair kernels only: the rows of every item this pass transforms (even bounds, all by default);
     // the others hold zeros that nobody reads (or writes, but for RF_ZERO_REST)
     int row_lo, row_hi;
     PassElems elems;
@@ -1554,6 +1554,9 @@ int row_candidates(int n, int* out);
 int pass_radices(int n, bool row, int variant, int lines, int* out, int max_out);
 // The kernels used without tuning (CORO_AUTOTUNE=0, or sizes without candidates).
 int row_variant_default(int n);
+int col_box_rows(int n);
+bool row_takes_band(int n, int variant);
+bool col_takes_band(int n, int lines);
 // The kernel a pass with these settings launches: persistent (1) or not, and its lines.
 void describe_pass(int n, bool dbl, bool row, int variant, int lines, int* persistent, int* out_lines);
 

@@ -116,6 +116,13 @@ int col_lines_default(int n, bool dbl) {
     }
 }
 
+// Rows of a column box: what ColArgs.in_lo ... out_hi count (0: no bands).
+int col_box_rows(int n) { return mixed_pair_length(n) ? mpair::pair_tma_rows(n) : 256; }
+
+// Whether a pass on this kernel takes a band of rows (RowArgs.row_lo ..., ColArgs.in_lo ...).
+bool row_takes_band(int n, int variant) { return variant == 3 || (mixed_pair_length(n) && (variant < 0 || variant == 6)); }
+bool col_takes_band(int n, int lines) { return lines == -9 || (mixed_pair_length(n) && (lines == 0 || lines == -5)); }
+
 int row_variant_default(int n) { return mixed_pair_length(n) ? 6 : (n >= 1024 && n <= 4096) ? 3 : 0; }
 
 int col_candidates(int n, int* out) {

@@ -212,7 +212,7 @@ def test_pass_flops(ctx):
     assert all(x == 2 * one for x in f[1:-1])
 
 
-@pytest.mark.parametrize("n", [1024, 2048, 4096])
+@pytest.mark.parametrize("n", [1024, 2048, 4096, 1400, 2800, 4100])
 @pytest.mark.parametrize("r_first,r_mid,r_last", [(0.5, 0.13, 0.2), (0.02, 0.0, 0.49), (0.1, 0.3, 0.0)])
 def test_rows_left_out_behind_masks(ctx, n, r_first, r_mid, r_last):
     """A uniform beam through an aperture, a stop between two hops, and a last stop (radii in units of
