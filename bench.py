@@ -539,19 +539,20 @@ def coronagraph_bench(ctx, device, steps: int, warmup: int, precision: int, n_la
     per = plan.unit_times(steps)                      # [steps][6]
     plan.set_timing(0)
     plan.use_graph(False)
-    # dense complex MACs of the six GEMMs; the plan's own counts weigh them by the products its
-    # precision issues (3 split terms: 24 flops per complex MAC, EXT: 10 slice products, 80 flops)
+    # dense complex MACs of the six contractions; the plan's own counts (real multiply-adds on even /
+    # odd halves, a quarter of the complex ones) weigh them by the products its precision issues
+    # (3xTF32 3, 3xBF16 6, EXT 10; 8 flops each per complex MAC)
     cmac = 0.0
     for it in items:
         mo = it["m_occ"]
         cmac += n * mo * n + mo * mo * n + mo * n * mo + n * n * mo + n * md * n + md * md * n
-    per_cmac = 80.0 if precision == coro.MFT_EXT else 24.0
+    per_cmac = {coro.MFT_EXT: 80.0, coro.MFT_3XBF16: 48.0}.get(precision, 24.0)
     # what the support-aware plan computes: only K ranges / tiles inside the spot and stop
     useful_flops, issued_flops = plan.flops()
     gemm_ms = float(per[:, 1:].sum())                 # stages 1-5 are tensor-core GEMM launches
     achieved = useful_flops * steps / (gemm_ms / 1e3) / 1e12
     pk, src = tensor_peak("tf32" if precision == coro.MFT_3XTF32 else "bf16", device)
-    kernel = "tcx_cgemm_kernel" if precision == coro.MFT_EXT else "tc_cgemm_kernel"
+    kernel = "ft_gemm_kernel"
     out = {"value": B * steps / (total_ms / 1e3), "unit": "PSFs/s", "batch": B,
            "precision": PRECISION_NAMES[precision],
            "workload": "broadband_lyot: 21 wavelengths (500-600 nm) x 8 DM sinc probes, 1024^2 pupil, "
@@ -777,13 +778,14 @@ def coronagraph_fp64(ctx, device, steps: int = 3) -> dict:
     b.record(stream)
     torch.cuda.synchronize()
     ms = a.elapsed_time(b) / steps
-    # complex multiply-adds of the three MFTs (two GEMMs each), 8 real flops apiece
+    # complex multiply-adds of the three MFTs (two contractions each); on even / odd halves with real
+    # bases each costs a quarter of 8 real flops
     n, mo, md = w.n, w.m_occ, w.m_det
     cmac = (mo * n * n + mo * mo * n) * 2 + md * n * n + md * md * n
-    achieved = 8.0 * cmac / (ms * 1e-3) / 1e12
+    achieved = 2.0 * cmac / (ms * 1e-3) / 1e12
     fp64_peak = 1.25
     roof = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,
-            "flops_per_psf": 8.0 * cmac, "kernel": "zgemm_simt_kernel (split K)",
+            "flops_per_psf": 2.0 * cmac, "kernel": "fold_zgemm_kernel",
             "peak_source": "nominal GB300 FP64 rate (an FP64 FMA probe measured 1.19 TFLOP/s)"}
     return {"value": 1e3 / ms, "unit": "PSFs/s", "ms_per_psf": ms, "precision": "FP64 (complex128)", "roofline": roof,
             "workload": "Lyot system of the broadband batch at its centre wavelength, one PSF per call sequence"}

@@ -323,8 +323,9 @@ coro_status coro_fresnel_plan_set_pass_kernel(coro_plan plan, int row_variant, i
  * rounding order. A plan starts on neither: at creation it takes the natural passes its tuner
  * picked, or (when faster, and without tuning) the packed-pair kernels with row pairs held
  * sample by sample interleaved between passes, in place, reported as layout 0; results are
- * bitwise those of the same kernels on the natural layout. The environment sets CORO_LAYOUT=0
- * to keep natural rows throughout, CORO_LAYOUT=1 for the alternating layout.
+ * bitwise those of the same kernels on the natural layout. There, and on the packed-pair engine
+ * of n = 1400, 2800, 4100, rows that apertures and stops make zero are left out. The environment
+ * sets CORO_LAYOUT=0 to keep natural rows throughout and every one of them, CORO_LAYOUT=1 for the alternating layout.
  * CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a
  * supported size. */
 coro_status coro_fresnel_plan_set_layout(coro_plan plan, int transposed);
@@ -369,12 +370,13 @@ coro_status coro_plan_destroy(coro_plan plan);
 typedef enum {
     CORO_MFT_FP32 = 0,    /* FP32 CUDA-core complex GEMM                                     */
     CORO_MFT_3XTF32 = 1,  /* split TF32 tensor-core GEMM (hi*hi + hi*lo + lo*hi), FP32 acc   */
-    CORO_MFT_3XBF16 = 2,  /* split BF16 tensor-core GEMM, FP32 accumulate                    */
+    CORO_MFT_3XBF16 = 2,  /* split BF16 tensor-core GEMM, FP32 accumulate (three planes, six */
+                          /* products; two planes, three products in complex GEMMs)          */
     CORO_MFT_FP64 = 3,    /* complex128 fields, FP64 CUDA-core GEMM (reference precision)    */
     CORO_MFT_EXT = 4      /* extended precision on the BF16 tensor cores: each operand value  */
-                          /* as four 8-bit slices of a power-of-two scale shared by 32       */
+                          /* as four 8-bit slices of a power-of-two scale shared by 64       */
                           /* consecutive K elements (32 bits), ten slice products summed     */
-                          /* exactly per 32-element group, two-float accumulation across     */
+                          /* exactly per 64-element group, two-float accumulation across     */
                           /* groups and in the epilogues; complex64 in and out               */
 } coro_mft_prec;
 
@@ -405,11 +407,13 @@ coro_status coro_dm_correlate(coro_ctx ctx, const float* w, int batch, int n, do
  *   E_det = MFT(E_D; m_det, du_det)
  *   I = |E_det|^2 / peak[b],   S[b] = sum of I over dh_in <= rho <= dh_out (lambda/D)
  * MFT conventions as in coro_propagate_mft (pupil pixel centre n/2, npix pixels across D).
- * Six split-precision tensor-core GEMMs over the whole batch; spot, Babinet subtraction, Lyot
- * stop, intensity and dark-hole sum are fused into GEMM epilogues. Items may have different
+ * Six split-precision tensor-core GEMMs over the whole batch, on the even and odd halves of every
+ * plane with real bases (a quarter of the complex products; planes trimmed to the spot and the
+ * stop); spot, Babinet subtraction and Lyot stop are fused into GEMM epilogues, intensity and
+ * dark-hole sum into the kernel that leaves the halves. Where a mask reaches the unpaired sample of
+ * an even axis (index 0, coordinate -n/2), complex GEMMs with the intensity fused run instead. Items may have different
  * occulter sizes m_occ (uneven per-wavelength sampling); n, npix, lyot_frac, m_det are shared.
- * The plan owns its work buffers (bases, split operands, about 80 MB per item at n = 1024 with
- * TF32) for its lifetime.
+ * The plan owns its work buffers (bases, split operands) for its lifetime.
  * ------------------------------------------------------------------------------------------ */
 typedef struct {
     int m_occ;            /* occulter samples per axis, [16, 8192]                          */
@@ -450,18 +454,22 @@ coro_status coro_lyot_plan_execute_n(coro_plan plan, const void* pupil, const do
  * (E_D = E_A . Lyot stop). Synchronises the stream. */
 coro_status coro_lyot_plan_peak(coro_plan plan, const void* pupil, double* peak_out);
 /* Run stages [first, first + count) only (for per-launch timing): 0 split of the pupil, 1-4 the
- * GEMMs pupil->occulter (two), occulter->Lyot with Babinet (two), 5 the detector MFT with the
- * intensity epilogue (two launches, preceded by one stream memset of the dark-hole sums).
+ * GEMMs pupil->occulter (two), occulter->Lyot with Babinet (two), 5 the detector MFT with its
+ * intensity (two GEMMs and, on halves, the kernel that leaves them; a stream memset of the
+ * dark-hole sums comes first).
  * Running 0-5 in order equals coro_lyot_plan_execute without the host copy of dh. */
 coro_status coro_lyot_plan_execute_range(coro_plan plan, const void* pupil, const double* peak, float* intensity,
                                          void* field, int first, int count);
-/* Tensor work of one execute (the six GEMMs), in flops: *useful = 24 per valid output per
- * complex product inside the operands' known support (the spot, the Lyot stop: the plan runs
- * only the K ranges and tiles those leave non-zero); *issued = the same over every 128 x 128
- * tile and K slice the kernels run (padding included). Either pointer may be NULL. Host only. */
+/* Tensor work of one execute (the six GEMMs), in flops: *useful = 2 per split product (3 for
+ * 3XTF32, 6 for 3XBF16, 10 for EXT) of every real multiply-add for a valid output inside the
+ * operands' known support (the spot, the Lyot stop: the plan runs only the K ranges and tiles
+ * those leave non-zero); *issued = the same over every tile and K slice the kernels run (padding
+ * included). Plans on complex GEMMs count 4 real multiply-adds per complex one, and 3 products for
+ * 3XBF16. Either pointer may be NULL. Host only. */
 coro_status coro_lyot_plan_flops(coro_plan plan, double* useful, double* issued);
-/* Tensor-core GEMM output tile of the plan (rows x complex columns): 128 x 128 for 3XTF32 /
- * 3XBF16; 128 x 64 or 128 x 32 for EXT, chosen when the plan is created by timing the plan's
+/* Tensor-core GEMM output tile of the plan (rows x complex columns; on halves EXT tiles have twice
+ * as many real columns, 3XTF32 / 3XBF16 tiles up to 128): 128 x 128 for 3XTF32 / 3XBF16;
+ * 128 x 64 or 128 x 32 for EXT, chosen when the plan is created by timing the plan's
  * GEMM stages at both widths (unless the environment sets CORO_AUTOTUNE=0, which keeps 64);
  * 0 x 0 for FP64 plans (CUDA-core GEMMs). Either pointer may be NULL. Host query. */
 coro_status coro_lyot_plan_gemm_tile(coro_plan plan, int* tile_m, int* tile_n);
@@ -508,8 +516,8 @@ typedef struct {
     const coro_lyot_item* items;  /* host [batch], one Lyot item per wavelength            */
     int precision;                /* CORO_MFT_3XTF32, CORO_MFT_3XBF16 or CORO_MFT_EXT      */
     int max_resident;             /* wavelengths held in HBM at once (3 x 8 n_fresnel^2    */
-                                  /* bytes each, 5 x where the Fresnel plans may take the  */
-                                  /* alternating layout: n_fresnel 1024 ... 4096); 0 = as  */
+                                  /* bytes each, 5 x at n_fresnel 1024 ... 4096, room for  */
+                                  /* the alternating layout's planes); 0 = as              */
                                   /* many as fit in 70 % of the free                       */
                                   /* device memory. The band runs in chunks of that many,  */
                                   /* with the same results (per-item sums in item order).  */

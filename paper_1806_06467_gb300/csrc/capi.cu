@@ -686,15 +686,15 @@ int interleaved_ops(int dtype, int n, std::vector<Op>& nat, std::vector<Op>* out
     return found;
 }
 
-// Rows that cannot matter are left out of interleaved passes and of the mixed-radix packed-pair ones: behind a mask (an aperture or stop) only
-// the rows it leaves are transformed, written before it by the column pass and read after it by the
-// next one, in boxes of 256 rows (mixed radix: 200 or 2 x 205); a plan's last row pass fills its other rows with zeros. first_in: rows
-// n/2 +- first_in are all the input's non-zeros (-1: unknown); last_out: only rows n/2 +- last_out of the
-// result are wanted (-1: all; the others are then left as they are). The first plane's mask counts
-// where the plan makes the field itself (INIT_ONE), so that what a caller's field holds under the mask
-// reaches the passes as before. Skipped are products with zeros: values are unchanged. 4096^2 relay
-// with a 1024-pixel pupil and stop: first pass 56 -> 29 us, last 53 -> 31, 828 -> 770 in all; 2800^2
-// with 700 pixels 689 -> 630.
+// Rows that cannot matter are left out of interleaved passes and of the mixed-radix packed-pair ones:
+// behind a mask (an aperture or stop) only the rows it leaves are transformed, written before it by the
+// column pass and read after it by the next one, in boxes of 256 rows (mixed radix: 200 or 2 x 205); a
+// plan's last row pass fills its other rows with zeros. first_in: rows n/2 +- first_in are all the
+// input's non-zeros (-1: unknown); last_out: only rows n/2 +- last_out of the result are wanted (-1: all;
+// the others are then left as they are). The first plane's mask counts where the plan makes the field
+// itself (INIT_ONE), so that what a caller's field holds under the mask reaches the passes as before.
+// Skipped are products with zeros: values are unchanged. 4096^2 relay with a 1024-pixel pupil and stop:
+// first pass 56 -> 29 us, last 53 -> 31, 828 -> 770 in all; 2800^2 with 700 pixels 689 -> 630.
 struct RowLimits {
     int first_in = -1, last_out = -1;
     bool internal = false;                // maps and stores are the library's own (wfc.cu)
