@@ -578,10 +578,12 @@ ft_fold_kernel(const float2* __restrict__ src, long long sb, int sld, int n, int
 
 template <int FMT>
 __global__ void __launch_bounds__(128)
-ft_basis_kernel(double c, int K, typename FtElem<FMT>::type* w, int R, int ld) {
+ft_basis_kernel(double c, const FtItem* __restrict__ items, int K, typename FtElem<FMT>::type* w, long long stride, int R, int ld) {
     constexpr bool EXT = FMT == FT_EXT;
     __shared__ uint32_t sh[EXT ? 2 : 1][4];
     const int k = blockIdx.x * 128 + threadIdx.x, n = blockIdx.y;
+    if (items) c = items[blockIdx.z].scale;
+    w += blockIdx.z * stride;
     double s = 0.0, co = 0.0;
     if (k < K) {
         double cyc = (double)((long long)k * n) * c;
@@ -908,14 +910,23 @@ cudaError_t ft_fold(int fmt, const float2* src, long long sb, int sld, int n, in
     return cudaGetLastError();
 }
 
-cudaError_t ft_basis(int fmt, double c, int K, int N, const FtOperand& w, int index, cudaStream_t stream) {
-    if (K > w.ld || N > w.R || index < 0 || index >= w.items) return cudaErrorInvalidValue;
-    const dim3 grid((w.ld + 127) / 128, N);
-    const size_t at = (size_t)index * w.stride;
-    if (fmt == FT_TF32) ft_basis_kernel<FT_TF32><<<grid, 128, 0, stream>>>(c, K, (float*)w.base + at, w.R, w.ld);
-    else if (fmt == FT_BF16) ft_basis_kernel<FT_BF16><<<grid, 128, 0, stream>>>(c, K, (__nv_bfloat16*)w.base + at, w.R, w.ld);
-    else ft_basis_kernel<FT_EXT><<<grid, 128, 0, stream>>>(c, K, (__nv_bfloat16*)w.base + at, w.R, w.ld);
+static cudaError_t basis_launch(int fmt, double c, const FtItem* items, int K, int N, const FtOperand& w, int first, int count,
+                                cudaStream_t stream) {
+    if (K > w.ld || N > w.R || first < 0 || first + count > w.items) return cudaErrorInvalidValue;
+    const dim3 grid((w.ld + 127) / 128, N, count);
+    const size_t at = (size_t)first * w.stride;
+    if (fmt == FT_TF32) ft_basis_kernel<FT_TF32><<<grid, 128, 0, stream>>>(c, items, K, (float*)w.base + at, w.stride, w.R, w.ld);
+    else if (fmt == FT_BF16) ft_basis_kernel<FT_BF16><<<grid, 128, 0, stream>>>(c, items, K, (__nv_bfloat16*)w.base + at, w.stride, w.R, w.ld);
+    else ft_basis_kernel<FT_EXT><<<grid, 128, 0, stream>>>(c, items, K, (__nv_bfloat16*)w.base + at, w.stride, w.R, w.ld);
     return cudaGetLastError();
+}
+
+cudaError_t ft_basis(int fmt, double c, int K, int N, const FtOperand& w, int index, cudaStream_t stream) {
+    return basis_launch(fmt, c, nullptr, K, N, w, index, 1, stream);
+}
+
+cudaError_t ft_bases(int fmt, const FtItem* items, int K, int N, const FtOperand& w, cudaStream_t stream) {
+    return basis_launch(fmt, 0.0, items, K, N, w, 0, w.items, stream);
 }
 
 size_t ft_plane_parts(int m) {

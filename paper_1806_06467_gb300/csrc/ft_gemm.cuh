@@ -99,6 +99,9 @@ cudaError_t ft_fold(int fmt, const float2* src, long long src_bstride, int src_l
                     const FtOperand& dst, cudaStream_t stream);
 // basis `index` of w: W[p][n][k] = cos / sin(2 pi c k n), n < N, k < K
 cudaError_t ft_basis(int fmt, double c, int K, int N, const FtOperand& w, int index, cudaStream_t stream);
+// All of w at once, c = items[index].scale (device). One launch: six of 221 x 58 one by one cost an MFT
+// 114^2 -> 440^2 of six fields 12 of its 74 us.
+cudaError_t ft_bases(int fmt, const FtItem* items, int K, int N, const FtOperand& w, cudaStream_t stream);
 
 // Classes T [item][px][py][c][R][ld] (FT_FLOAT of two GEMMs; v rows, u columns) to the plane: field =
 // scale F, intensity |scale F|^2 inv_peak, its sum over lo <= r^2 <= thr_out, its largest value.

@@ -63,7 +63,7 @@ coro_status mft_tensor_core(coro_ctx ctx, const coro_wavefront* in, int directio
     if (!it) return st;
     FtGemm g1, g2;
     cudaError_t e = ft_fold(fmt, (const float2*)in->data, (long long)n * n, n, n, hn, -1, X, ctx->stream);
-    for (int b = 0; b < batch && e == cudaSuccess; ++b) e = ft_basis(fmt, c[b], hn, hm, W, b, ctx->stream);
+    if (e == cudaSuccess) e = ft_bases(fmt, it + 2 * batch, hn, hm, W, ctx->stream);      // scale = c
     if (e == cudaSuccess) e = ft_make(fmt, X, W, batch, hm, 128, &g1);
     if (e == cudaSuccess) e = ft_make(fmt, Y, W, batch, hm, 128, &g2);
     if (e == cudaSuccess) {
