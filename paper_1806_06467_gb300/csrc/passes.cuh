@@ -320,9 +320,12 @@ __device__ __forceinline__ void apply_elems_pair(pk::CP (&v)[16], int x0, int ya
     using pk::CP;
     using pk::u64;
     const int kya = ya - N / 2, kyb = kya + 1;
+    // A mask selects, as in apply_elems: what is not finite under it does not leave it (times 0 it would
+    // be NaN, and fill the field in the next transform). By bits of the packed pair: 4096^2 relay
+    // 779 us (776 as a product, 833 with selects on the unpacked halves, which take registers).
     auto mask = [&](int s, bool pa, bool pb) {
-        const u64 m = pk::pack(pa ? 1.f : 0.f, pb ? 1.f : 0.f);
-        v[s] = CP{pk::mul2(v[s].re, m), pk::mul2(v[s].im, m)};
+        const u64 m = (pa ? 0xffffffffull : 0ull) | (pb ? 0xffffffffull << 32 : 0ull);
+        v[s] = CP{v[s].re & m, v[s].im & m};
     };
     // v[s] *= (fr_a + i fi_a, fr_b + i fi_b)
     auto mulf = [&](int s, u64 fr, u64 fi) {
