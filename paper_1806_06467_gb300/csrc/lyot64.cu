@@ -271,6 +271,8 @@ coro_status lyot64_create(coro_ctx ctx, const coro_lyot_desc* d, coro_plan* out)
     if (e == cudaSuccess) e = cudaMalloc(&p->part, sizeof(double) * kFinishBlocks);
     if (e == cudaSuccess) e = cudaMalloc(&p->dh, sizeof(double) * p->batch);
     if (e == cudaSuccess) e = make_folds(p.get());
+    // the bases are there before the plan is: its executes may go to another stream
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p->ctx->stream);
     if (e != cudaSuccess) return cuda_fail(e, "coro_lyot_plan_create (FP64)");
     *out = p.release();
     return CORO_OK;

@@ -112,3 +112,30 @@ def test_lyot_tensor_core_halves(ctx, n, npix, frac, m_occ, spot, m_det, dh_out,
         assert rel_l2(fld[b].cpu().numpy(), det) < 1e-3
         assert rel_l2(g[b].cpu().numpy(), adjoint.lyot_adjoint(mask * det / pk, p)) < 1e-3
     plan.close()
+
+
+@pytest.mark.parametrize("prec", [coro.MFT_FP64, coro.MFT_3XTF32])
+def test_lyot_plan_runs_on_a_stream_set_after_its_creation(lib, prec):
+    """A plan made behind long work on the context's first stream, executed on another stream at once:
+    its bases are complete when creation returns."""
+    n, md = 128, 96
+    items = [dict(m_occ=40, du_occ=0.25, spot_radius=3.0, du_det=0.5, dh_in=4.0, dh_out=11.0)]
+    e = coronagraph.pupil_field(n, 120.0, 550e-9, None)[None]
+    x = torch.from_numpy(e.astype(np.complex128 if prec == coro.MFT_FP64 else np.complex64)).cuda()
+    img = [torch.empty((1, md, md), dtype=torch.float32, device="cuda") for _ in range(2)]
+    busy = torch.ones((4096, 4096), device="cuda")
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    for k in range(2):
+        c = coro.Context(0, stream=first)
+        torch.cuda.synchronize()
+        if k:
+            with torch.cuda.stream(first):
+                for _ in range(40):
+                    busy = (busy @ busy).clamp_(0.0, 1.0)
+        plan = coro.LyotPlan(c, n=n, npix=120.0, lyot_frac=0.8, m_det=md, items=items, precision=prec)
+        if k:
+            c.lib.check(c.lib.coro_ctx_set_stream(c.handle, second.cuda_stream))
+        plan.execute(x, peak=1.0, intensity=img[k], want_dh=False)
+        torch.cuda.synchronize()
+        plan.close()
+    assert torch.equal(img[0], img[1])
