@@ -654,8 +654,8 @@ struct Op {
     const void* tab_x = nullptr;
     const void* tab_y = nullptr;
     // rows that a mask of this (row) pass leaves: n/2 - mask_r ... n/2 + mask_r; -1: no mask. mask_map /
-    // mask_store: a map after the mask (its infinities would leave the mask), an element that writes
-    // to caller memory
+    // mask_store: an element after the mask whose factors need not be finite (0 times them is NaN, which
+    // left-out rows would not show), an element that writes to caller memory
     int mask_r = -1;
     bool mask_map = false, mask_store = false;
     // the rows and boxes that the pass runs (RowArgs, ColArgs); hi = 0: all
@@ -1212,6 +1212,20 @@ coro_status qpf_elem(DevBlocks& db, bool dbl, int n, int batch, const double* ps
     return out->tab ? CORO_OK : st;
 }
 
+// Whether every factor of an element is known to be finite in the field's 32 bits: not a map's (its
+// values are the caller's, read on the device), nor that of parameters that overflow on the way.
+bool bounded_factor(const coro_element* el, const std::vector<double>& ps, const double* lam, int batch) {
+    auto small = [](double v) { return std::fabs(v) < 1e30; };
+    bool ok = el->kind != CORO_EL_OPD_MAP && (el->kind != CORO_EL_SCALAR || small(el->scalar));
+    for (int b = 0; b < batch && ok; ++b) {
+        if (el->kind == CORO_EL_LENS) ok = small(ps[b] * ps[b] / (2.0 * lam[b] * el->focal_length));
+        if (el->kind == CORO_EL_SINE) ok = small(2.0 * el->sine_amplitude / lam[b]) && small(el->sine_freq * ps[b]);
+        if (el->kind == CORO_EL_ZERNIKE)
+            for (int i = 0; i < el->n_coeffs; ++i) ok = ok && small(2e3 * el->coeffs[i] / lam[b]);   // polynomials of order 7 stay below 1e3
+    }
+    return ok;
+}
+
 // Compile planes and hops into row / column passes (the fused pass scheduler shared by the
 // explicit and the pilot-beam plan builders).
 coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0, const double* lam,
@@ -1253,7 +1267,7 @@ coro_status build_passes(FresnelPlan* plan, int n, int batch, const double* ps0,
                 }
                 mask_r = mask_r < 0 ? r : std::min(mask_r, r);
             }
-            mask_map = mask_map || (mask_r >= 0 && el->kind == CORO_EL_OPD_MAP);
+            mask_map = mask_map || (mask_r >= 0 && !bounded_factor(el, ps, lam, batch));
             mask_store = mask_store || el->kind == CORO_EL_CHECKPOINT || el->kind == CORO_EL_PHASE_GRAD;
             // after an angular-spectrum hop the row pass holds the field times (-1)^(x+y)
             // (the fftshift sign is carried into the next forward FFT); checkpoints undo it

@@ -60,3 +60,24 @@ def test_samples_under_masks_that_are_not_finite(ctx, n, layout, monkeypatch):
             plan.close()
     assert bool(torch.isfinite(torch.view_as_real(out[0])).all())
     assert torch.equal(out[2], out[0]) and torch.equal(out[3], out[1])
+
+
+@pytest.mark.parametrize("kw", [dict(kind=coro.EL_SCALAR, scalar=float("inf")), dict(kind=coro.EL_SCALAR, scalar=1e300),
+                                dict(kind=coro.EL_SINE, sine_freq=2.0, sine_amplitude=float("nan")),
+                                dict(kind=coro.EL_ZERNIKE, radius=1.0, coeffs=[1e-8, float("nan")], j_first=4)])
+def test_factors_behind_a_mask_that_are_not_finite(ctx, kw, monkeypatch):
+    """0 times an infinite or NaN factor is NaN: rows are not left out as zeros behind such an element."""
+    n = 1024
+    monkeypatch.setenv("CORO_AUTOTUNE", "0")
+    els = [coro.element(coro.EL_APERTURE, plane=0, radius=0.2), coro.element(coro.EL_CIRCLE, plane=1, radius=0.1),
+           coro.element(kw["kind"], plane=1, **{k: v for k, v in kw.items() if k != "kind"})]
+    out = []
+    for layout in (None, "0"):
+        monkeypatch.delenv("CORO_LAYOUT", raising=False) if layout is None else monkeypatch.setenv("CORO_LAYOUT", layout)
+        plan = coro.FresnelPlan(ctx, n=n, batch=1, pixelscale=1.0 / n, wavelength=550e-9, distances=[1.5], elements=els,
+                                init_uniform=True)
+        x = torch.empty((1, n, n), dtype=torch.complex64, device="cuda")
+        plan.execute(x)
+        out.append(torch.view_as_real(x))
+        plan.close()
+    assert bool(torch.isnan(out[1]).any()) and torch.equal(torch.isnan(out[0]), torch.isnan(out[1]))
