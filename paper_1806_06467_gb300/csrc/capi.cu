@@ -1836,21 +1836,23 @@ extern "C" coro_status coro_plan_destroy(coro_plan plan) {
 
 namespace {
 
-// (re^2 + im^2) / norm, rounded once: complex64 samples in two-float arithmetic (squares and their sum
-// exact to 2^-46, the product with 1 / norm = sh + sl alike), because FP64 runs at 1/64 of the FP32 rate
-// here: 2048^2 (50 MB) took 51 us in FP64, 12 us like this. Sums and results outside [1e-30, 1e30],
-// where a part would under- or overflow, take FP64.
-// (a call: predicated, its instructions would occupy the FP64 pipe for every sample)
+// (re^2 + im^2) / norm of complex64 samples, the bits of FP64 arithmetic rounded once, without FP64 for nearly
+// all of them: FP64 runs at 1/64 of the FP32 rate here (2048^2, 50 MB: 51 us in FP64, 14 like this).
+// Two-float arithmetic is off by less than 2^-44 of the result (squares exact, their sum and the products
+// with 1 / norm = sh + sl to 2^-46 or so each): where +- 2^-43 round alike, so does FP64. The others, one in
+// some 2^18, take FP64, and so do sums and results outside [1e-30, 1e30], where a part would under- or
+// overflow, or a value be none. (A call: predicated, its instructions would occupy the FP64 pipe for every sample.)
 __device__ __noinline__ float intensity_fp64(float2 v, double s) { return (float)(((double)v.x * v.x + (double)v.y * v.y) * s); }
 
 __device__ __forceinline__ float intensity_of(float2 v, double s, float sh, float sl) {
     const float p = v.x * v.x, q = v.y * v.y, h = p + q;
     if (v.x == 0.f && v.y == 0.f) return 0.f;            // outside a stop; s is finite
     const float r = h * sh;
-    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f)) return intensity_fp64(v, s);
     const float ep = fmaf(v.x, v.x, -p), eq = fmaf(v.y, v.y, -q), bb = h - p;
     const float l = ((p - (h - bb)) + (q - bb)) + (ep + eq);
-    return r + (fmaf(h, sh, -r) + (h * sl + l * sh));
+    const float t = fmaf(h, sh, -r) + (h * sl + l * sh), up = r + fmaf(r, 0x1p-43f, t);
+    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f && up == r + fmaf(r, -0x1p-43f, t))) return intensity_fp64(v, s);
+    return up;
 }
 
 // grid.y: items. Two samples per thread and step where they sit on a 16-byte boundary.

@@ -581,3 +581,29 @@ def test_intensity_rounds_once_over_the_whole_range(ctx, n, batch):
         assert np.all(np.abs(got[fin] - ref[fin]) <= 0.5001 * np.spacing(ref32[fin]))          # half a unit
         assert np.array_equal(got[~np.isfinite(ref32)], ref32[~np.isfinite(ref32)], equal_nan=True)
         assert np.all(got[ref == 0.0] == 0.0)
+
+
+@pytest.mark.parametrize("norm", [1.0, 3.7, 8.1e4])
+def test_intensity_bits_next_to_ties(ctx, norm):
+    """Samples whose FP64 intensity lies within 2^-44 of the middle between two floats, picked out of
+    2^28: the bits of FP64 arithmetic rounded once."""
+    g = torch.Generator(device="cuda").manual_seed(int(norm))
+    inv = 1.0 / norm
+    picked = []
+    for _ in range(16):
+        v = torch.randn((1 << 24, 2), generator=g, device="cuda")
+        w = v.double()
+        e = (w[:, 0] * w[:, 0] + w[:, 1] * w[:, 1]) * inv
+        low = e.view(torch.int64) & ((1 << 29) - 1)
+        picked.append(v[(low - (1 << 28)).abs() < (1 << 8)])
+    v = torch.cat(picked)
+    n = 32
+    assert len(v) > 100
+    v = v[:n * n]
+    f = torch.ones((n * n, 2), device="cuda")
+    f[:len(v)] = v
+    out = torch.empty((1, n, n), dtype=torch.float32, device="cuda")
+    coro.intensity(ctx, torch.view_as_complex(f).reshape(1, n, n), norm=[norm], out=out)
+    x = f.cpu().numpy().astype(np.float64)
+    ref = ((x[:, 0] ** 2 + x[:, 1] ** 2) * inv).astype(np.float32)
+    np.testing.assert_array_equal(out.cpu().numpy().reshape(-1), ref)
