@@ -365,7 +365,8 @@ coro_status coro_plan_destroy(coro_plan plan);
  * in: [batch][n_in][n_in]; out: [batch][m][m], both C64 (precisions FP32 / 3XTF32 / 3XBF16 / EXT) or
  * both C128 (precision FP64). du: host [batch] (lambda/D per pixel of the focal-plane side).
  * npix: pupil pixels across D. precision: coro_mft_prec.
- * Work buffers are taken from the context (allocated on first use, grown as needed).
+ * Work buffers are taken from the context (allocated on first use, grown as needed); a large batch
+ * runs in rounds, so that they stay within 2 GiB where one item's are smaller than that.
  * ------------------------------------------------------------------------------------------ */
 typedef enum {
     CORO_MFT_FP32 = 0,    /* FP32 CUDA-core complex GEMM                                     */

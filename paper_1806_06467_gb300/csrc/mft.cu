@@ -5,8 +5,9 @@
 //   out = s * A_y . in . A_x^T,   A[u][j] = exp(-+ 2 pi i X_j U_u)
 //
 // evaluated as two batched GEMMs over even / odd halves with real bases: on the CUDA cores
-// (fold.cuh) or on the tensor cores (ft_gemm.cuh). The bases are generated on the device in FP64 (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64
-// constant, reduced to its fractional cycle before sincospi) and rounded.
+// (fold.cuh) or on the tensor cores (ft_gemm.cuh). The bases are generated on the device in FP64
+// (the phase X_j U_u = j' u' du / npix is an exact integer times one FP64 constant, reduced to its
+// fractional cycle before sincospi) and rounded.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,82 +32,105 @@ coro_status check_mft_wf(const char* fn, const coro_wavefront* wf) {
     return CORO_OK;
 }
 
+// Items of a batch that one round takes: their workspace stays within 2 GiB, or is that of one item.
+// (The classes of a plane are as large as the plane: a batch that fills most of the device would
+// otherwise need as much again. Rounds of 2 GiB are far past what fills the chip.)
+int round_items(int batch, size_t item_bytes, int most) {
+    const size_t fit = ((size_t)2 << 30) / item_bytes;
+    return (int)std::max<size_t>(1, std::min<size_t>({fit, (size_t)batch, (size_t)most}));
+}
+
 // Tensor-core MFT (3xTF32, 3xBF16, EXT) on even / odd halves (ft_gemm.cuh): fold, bases, two
 // contractions to the parity classes of the result, and the plane of all signs.
 coro_status mft_tensor_core(coro_ctx ctx, const coro_wavefront* in, int direction, int m, const std::vector<double>& c,
                             int fmt, coro_wavefront* out) {
     coro_status st = CORO_OK;
-    const int batch = in->batch, n = in->n, hn = fold_len(n), hm = fold_len(m);
-    FtOperand X = ft_operand(fmt, batch, hn, hn), W = ft_basis_operand(fmt, batch, hm, hn), Y = ft_operand(fmt, batch, hm, hn);
-    const int ld_t = ft_pitch(FT_TF32, hm);
-    const size_t t_bytes = (size_t)batch * 8 * hm * ld_t * (fmt == FT_EXT ? sizeof(float2) : sizeof(float));
+    const int n = in->n, hn = fold_len(n), hm = fold_len(m), ld_t = ft_pitch(FT_TF32, hm);
+    const size_t t_item = (size_t)8 * hm * ld_t * (fmt == FT_EXT ? sizeof(float2) : sizeof(float));
     auto align = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
-    const size_t xb = align(ft_bytes(fmt, X)), wb = align(ft_bytes(fmt, W)), yb = align(ft_bytes(fmt, Y));
-    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, xb + wb + yb + t_bytes, &st);
+    FtOperand X, W, Y;
+    // T, written when X has been read, takes its place
+    size_t xb, wb, yb;
+    auto shape = [&](int items) {
+        X = ft_operand(fmt, items, hn, hn);
+        W = ft_basis_operand(fmt, items, hm, hn);
+        Y = ft_operand(fmt, items, hm, hn);
+        xb = align(std::max(ft_bytes(fmt, X), t_item * items));
+        wb = align(ft_bytes(fmt, W));
+        yb = align(ft_bytes(fmt, Y));
+    };
+    shape(1);
+    const int round = round_items(in->batch, xb + wb + yb, in->batch);
+    shape(round);
+    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, xb + wb + yb, &st);
     if (!work) return st;
-    X.base = work;
-    W.base = work + xb;
-    Y.base = work + xb + wb;
-    void* T = work + xb + wb + yb;
-    std::vector<FtItem> items(batch);
-    for (int b = 0; b < batch; ++b) items[b] = FtItem{hn, hm, 0, b, -1, 0x7fffffff, 0, 1.0, 1.0};
-    std::vector<FtItem> both(items);
-    both.insert(both.end(), items.begin(), items.end());
-    for (int b = 0; b < batch; ++b) {
-        both[b].H = hn;                              // rows: k of the other axis, then u
-        both[batch + b].H = hm;
+    for (int b0 = 0; b0 < in->batch; b0 += round) {
+        const int batch = std::min(round, in->batch - b0);
+        shape(batch);
+        X.base = work;
+        W.base = work + xb;
+        Y.base = work + xb + wb;
+        void* T = work;
+        std::vector<FtItem> items(batch);
+        for (int b = 0; b < batch; ++b) items[b] = FtItem{hn, hm, 0, b, -1, 0x7fffffff, 0, 1.0, 1.0};
+        std::vector<FtItem> both(items);
+        both.insert(both.end(), items.begin(), items.end());
+        for (int b = 0; b < batch; ++b) {
+            both[b].H = hn;                              // rows: k of the other axis, then u
+            both[batch + b].H = hm;
+        }
+        std::vector<FtItem> plane(items);
+        for (int b = 0; b < batch; ++b) plane[b].scale = c[b0 + b];
+        both.insert(both.end(), plane.begin(), plane.end());
+        FtItem* it = (FtItem*)coro::upload_async(ctx, both.data(), both.size() * sizeof(FtItem), &st);
+        if (!it) return st;
+        FtGemm g1, g2;
+        cudaError_t e = ft_fold(fmt, (const float2*)in->data + (size_t)b0 * n * n, (long long)n * n, n, n, hn, -1, X, ctx->stream);
+        if (e == cudaSuccess) e = ft_bases(fmt, it + 2 * batch, hn, hm, W, ctx->stream);      // scale = c
+        if (e == cudaSuccess) e = ft_make(fmt, X, W, batch, hm, 128, &g1);
+        if (e == cudaSuccess) e = ft_make(fmt, Y, W, batch, hm, 128, &g2);
+        if (e == cudaSuccess) {
+            FtArgs a{};
+            a.items = it;
+            a.err = ctx->err;
+            a.R = X.R;
+            a.dst = Y.base;
+            a.dst_bstride = Y.stride;
+            a.dst_R = Y.R;
+            a.dst_ld = Y.ld;
+            e = ft_launch(g1, FT_SPLIT, a, ctx->stream);
+        }
+        if (e == cudaSuccess) {
+            FtArgs a{};
+            a.items = it + batch;
+            a.err = ctx->err;
+            a.R = Y.R;
+            a.dst = T;
+            a.dst_bstride = (long long)8 * hm * ld_t;
+            a.dst_R = hm;
+            a.dst_ld = ld_t;
+            e = ft_launch(g2, FT_FLOAT, a, ctx->stream);
+        }
+        if (e == cudaSuccess) {
+            FtPlane p{};
+            p.items = it + 2 * batch;
+            p.T = T;
+            p.ext = fmt == FT_EXT;
+            p.R = hm;
+            p.ld = ld_t;
+            p.bstride = (long long)8 * hm * ld_t;
+            p.m = m;
+            p.sign = direction < 0 ? -1 : 1;
+            p.field = (float2*)out->data + (size_t)b0 * m * m;
+            e = ft_plane(p, batch, ctx->stream);
+        }
+        coro::free_async(ctx, it);
+        if (e == cudaErrorNotSupported) {
+            coro::set_error("coro_propagate_mft: tensor maps unavailable (driver entry point missing)");
+            return CORO_ENOTIMPL;
+        }
+        if (e != cudaSuccess) return coro::cuda_fail(e, "tensor-core MFT");
     }
-    std::vector<FtItem> plane(items);
-    for (int b = 0; b < batch; ++b) plane[b].scale = c[b];
-    both.insert(both.end(), plane.begin(), plane.end());
-    FtItem* it = (FtItem*)coro::upload_async(ctx, both.data(), both.size() * sizeof(FtItem), &st);
-    if (!it) return st;
-    FtGemm g1, g2;
-    cudaError_t e = ft_fold(fmt, (const float2*)in->data, (long long)n * n, n, n, hn, -1, X, ctx->stream);
-    if (e == cudaSuccess) e = ft_bases(fmt, it + 2 * batch, hn, hm, W, ctx->stream);      // scale = c
-    if (e == cudaSuccess) e = ft_make(fmt, X, W, batch, hm, 128, &g1);
-    if (e == cudaSuccess) e = ft_make(fmt, Y, W, batch, hm, 128, &g2);
-    if (e == cudaSuccess) {
-        FtArgs a{};
-        a.items = it;
-        a.err = ctx->err;
-        a.R = X.R;
-        a.dst = Y.base;
-        a.dst_bstride = Y.stride;
-        a.dst_R = Y.R;
-        a.dst_ld = Y.ld;
-        e = ft_launch(g1, FT_SPLIT, a, ctx->stream);
-    }
-    if (e == cudaSuccess) {
-        FtArgs a{};
-        a.items = it + batch;
-        a.err = ctx->err;
-        a.R = Y.R;
-        a.dst = T;
-        a.dst_bstride = (long long)8 * hm * ld_t;
-        a.dst_R = hm;
-        a.dst_ld = ld_t;
-        e = ft_launch(g2, FT_FLOAT, a, ctx->stream);
-    }
-    if (e == cudaSuccess) {
-        FtPlane p{};
-        p.items = it + 2 * batch;
-        p.T = T;
-        p.ext = fmt == FT_EXT;
-        p.R = hm;
-        p.ld = ld_t;
-        p.bstride = (long long)8 * hm * ld_t;
-        p.m = m;
-        p.sign = direction < 0 ? -1 : 1;
-        p.field = (float2*)out->data;
-        e = ft_plane(p, batch, ctx->stream);
-    }
-    coro::free_async(ctx, it);
-    if (e == cudaErrorNotSupported) {
-        coro::set_error("coro_propagate_mft: tensor maps unavailable (driver entry point missing)");
-        return CORO_ENOTIMPL;
-    }
-    if (e != cudaSuccess) return coro::cuda_fail(e, "tensor-core MFT");
     return CORO_OK;
 }
 
@@ -118,21 +142,24 @@ coro_status mft_cuda_cores(coro_ctx ctx, const coro_wavefront* in, int direction
     using R = typename real_of<C>::type;
     coro_status st = CORO_OK;
     const int batch = in->batch, n = in->n, hn = fold_len(n), hm = fold_len(m), ldw = fold_ldw(hm);
-    // items per round: the contractions carry item x parity (x K split) in grid z
-    const int round = batch < 4096 ? batch : 4096;
     auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
-    const size_t f_bytes = align((size_t)round * 4 * hn * hn * sizeof(C)), w_bytes = align((size_t)round * 2 * hn * ldw * sizeof(R));
-    const size_t y_bytes = align((size_t)round * 4 * hn * hm * sizeof(C)), t_bytes = align((size_t)round * 4 * hm * hm * sizeof(C));
+    // T, written when F has been read, takes its place
+    auto f_bytes = [&](size_t k) { return align(k * 4 * std::max((size_t)hn * hn, (size_t)hm * hm) * sizeof(C)); };
+    auto w_bytes = [&](size_t k) { return align(k * 2 * hn * ldw * sizeof(R)); };
+    auto y_bytes = [&](size_t k) { return align(k * 4 * hn * hm * sizeof(C)); };
+    // the contractions carry item x parity (x K split) in grid z: 4096 items at most
+    const int round = round_items(batch, f_bytes(1) + w_bytes(1) + y_bytes(1), 4096);
+    const int rest = batch % round ? batch % round : round;       // items of the last round: other K splits
     size_t part_elems = 0;
     if (std::is_same<C, float2>::value)
-        part_elems = std::max(fold_part_elems(2 * hn, hm, hn, round), fold_part_elems(2 * hm, hm, hn, round));
-    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, f_bytes + w_bytes + y_bytes + t_bytes + part_elems * sizeof(C), &st);
+        for (int k : {round, rest})
+            part_elems = std::max({part_elems, fold_part_elems(2 * hn, hm, hn, k), fold_part_elems(2 * hm, hm, hn, k)});
+    unsigned char* work = (unsigned char*)coro::ctx_work(ctx, f_bytes(round) + w_bytes(round) + y_bytes(round) + part_elems * sizeof(C), &st);
     if (!work) return st;
-    C* F = (C*)work;
-    R* W = (R*)(work + f_bytes);
-    C* Y = (C*)(work + f_bytes + w_bytes);
-    C* T = (C*)(work + f_bytes + w_bytes + y_bytes);
-    C* part = part_elems ? (C*)(work + f_bytes + w_bytes + y_bytes + t_bytes) : nullptr;
+    C *F = (C*)work, *T = F;
+    R* W = (R*)(work + f_bytes(round));
+    C* Y = (C*)(work + f_bytes(round) + w_bytes(round));
+    C* part = part_elems ? (C*)(work + f_bytes(round) + w_bytes(round) + y_bytes(round)) : nullptr;
     cudaError_t e = cudaSuccess;
     for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += round) {
         const int nb = std::min(round, batch - b0);

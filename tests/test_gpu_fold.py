@@ -139,3 +139,23 @@ def test_lyot_plan_runs_on_a_stream_set_after_its_creation(lib, prec):
         torch.cuda.synchronize()
         plan.close()
     assert torch.equal(img[0], img[1])
+
+
+@pytest.mark.parametrize("prec", sorted(TOL))
+def test_mft_workspace_is_bounded(lib, prec):
+    """A batch whose classes would take more than 2 GiB runs in rounds: no more device memory than that is
+    taken, and items of every round are the oracle's (the last round is a ragged one)."""
+    n, m, batch = 32, 1024, 300
+    c = coro.Context(0)
+    x = torch.from_numpy(inputs.random_field((batch, n, n), seed=5).astype(np.complex128 if prec == coro.MFT_FP64 else np.complex64)).cuda()
+    du = np.linspace(0.1, 0.4, batch)
+    coro.propagate_mft(c, x[:1].contiguous(), float(n), -1, m, du[:1], prec)         # modules loaded
+    torch.cuda.synchronize()
+    out = torch.empty((batch, m, m), dtype=x.dtype, device="cuda")
+    before = torch.cuda.mem_get_info()[0]
+    coro.propagate_mft(c, x, float(n), -1, m, du, prec, out=out)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= (2 << 30) + (64 << 20)
+    for b in (0, 57, 121, 122, 150, 243, 298, 299):
+        assert rel_l2(out[b].cpu().numpy(), propagation.mft(x[b].cpu().numpy().astype(np.complex128), float(n), m, du[b])) < TOL[prec]
+    c.close()
