@@ -249,25 +249,51 @@ ft_gemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
                     tc::tc_fence_after();
                     const uint32_t d0 = tbase + buf * BUF;
                     const uint32_t xa = tc::smem_u32(smem + s * stage_bytes), wa = xa + x_bytes;
+                    const uint32_t keep = first ? 0u : 1u;
+                    if constexpr (EXT) {
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {             // two MMA K steps of 32 bytes
-                        // plane and K-step offsets move the descriptor's start address only
-                        const uint64_t dx = tc::sdesc_sw128(xa + kk * 32), dw = tc::sdesc_sw128(wa + kk * 32);
-                        const uint32_t keep = first && kk == 0 ? 0u : 1u;
+                        for (int kk = 0; kk < 2; ++kk) {             // two MMA K steps of 32 bytes
+                            // plane and K-step offsets move the descriptor's start address only
+                            const uint64_t dx = tc::sdesc_sw128(xa + kk * 32), dw = tc::sdesc_sw128(wa + kk * 32);
 #pragma unroll
-                        for (int i = 0; i < S; ++i) {
-                            const uint64_t ad = dx + (uint64_t)(((i >> 1) * XPAIR_BYTES + (i & 1) * 64) >> 4);
-                            const int last = S - 1 - i;          // products of planes i + j < S
+                            for (int i = 0; i < S; ++i) {
+                                const uint64_t ad = dx + (uint64_t)(((i >> 1) * XPAIR_BYTES + (i & 1) * 64) >> 4);
+                                const int last = S - 1 - i;          // products of planes i + j < S
 #pragma unroll
-                            for (int j = 0; j <= last; ++j) {
-                                const uint64_t bd = dw + (uint64_t)(((j >> 1) * wpair + (j & 1) * 64) >> 4);
-                                // FT_EXT: level 0 alone, levels 1-3 in a second accumulator
-                                const uint32_t d = d0 + (EXT && i + j ? 128u : 0u);
-                                const uint32_t acc = (i == 0 && j <= (EXT ? 1 : 0)) ? keep : 1u;
-                                if (last == 0) tc::umma_coll<Cfg::B16, tc::COLL_NONE>(d, ad, bd, ID, acc);
-                                else if (j == 0) tc::umma_coll<Cfg::B16, tc::COLL_FILL>(d, ad, bd, ID, acc);
-                                else if (j == last) tc::umma_coll<Cfg::B16, tc::COLL_LASTUSE>(d, ad, bd, ID, acc);
-                                else tc::umma_coll<Cfg::B16, tc::COLL_USE>(d, ad, bd, ID, acc);
+                                for (int j = 0; j <= last; ++j) {
+                                    const uint64_t bd = dw + (uint64_t)(((j >> 1) * wpair + (j & 1) * 64) >> 4);
+                                    // level 0 alone, levels 1-3 in a second accumulator
+                                    const uint32_t d = d0 + (i + j ? 128u : 0u);
+                                    const uint32_t acc = kk == 0 && i == 0 && j <= 1 ? keep : 1u;
+                                    if (last == 0) tc::umma_coll<Cfg::B16, tc::COLL_NONE>(d, ad, bd, ID, acc);
+                                    else if (j == 0) tc::umma_coll<Cfg::B16, tc::COLL_FILL>(d, ad, bd, ID, acc);
+                                    else if (j == last) tc::umma_coll<Cfg::B16, tc::COLL_LASTUSE>(d, ad, bd, ID, acc);
+                                    else tc::umma_coll<Cfg::B16, tc::COLL_USE>(d, ad, bd, ID, acc);
+                                }
+                            }
+                        }
+                    } else {
+                        // products with the lower planes of X first, those of its upper plane from the lowest
+                        // plane of W up: every MMA cuts its sum off at the accumulator's last bit, so the
+                        // small products go in while it is small (dark-hole sums of 3xTF32 Lyot images off
+                        // by 1.6e-5 with the products from large to small, 1.2e-5 like this; 3xBF16 1.4e-5
+                        // and 0.5e-5; same time)
+                        const uint64_t dx = tc::sdesc_sw128(xa), dw = tc::sdesc_sw128(wa);
+#pragma unroll
+                        for (int i = S - 1; i >= 0; --i) {
+                            const uint64_t di = dx + (uint64_t)(((i >> 1) * XPAIR_BYTES + (i & 1) * 64) >> 4);
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                const uint64_t ad = di + kk * 2;
+#pragma unroll
+                                for (int j = S - 1 - i; j >= 0; --j) {
+                                    const uint64_t bd = dw + (uint64_t)(((j >> 1) * wpair + (j & 1) * 64) >> 4) + kk * 2;
+                                    const uint32_t acc = kk == 0 && i == S - 1 ? keep : 1u;
+                                    if (i == S - 1) tc::umma_coll<Cfg::B16, tc::COLL_NONE>(d0, ad, bd, ID, acc);
+                                    else if (j == S - 1 - i) tc::umma_coll<Cfg::B16, tc::COLL_FILL>(d0, ad, bd, ID, acc);
+                                    else if (j == 0) tc::umma_coll<Cfg::B16, tc::COLL_LASTUSE>(d0, ad, bd, ID, acc);
+                                    else tc::umma_coll<Cfg::B16, tc::COLL_USE>(d0, ad, bd, ID, acc);
+                                }
                             }
                         }
                     }

@@ -325,3 +325,34 @@ def test_broadband_batch_sampled_items(ctx, prec):
         assert err < DH_TOL_FULL[prec]
         assert np.max(np.abs(got - ref_i)) < 1e-5
     plan.use_graph(False)
+
+
+@pytest.mark.parametrize("prec,bar", [(coro.MFT_3XTF32, 1.46e-5), (coro.MFT_3XBF16, 1.44e-5)])
+def test_darkhole_sums_are_as_close_as_with_complex_products(ctx, prec, bar):
+    """Relative error (RMS over the items) of the dark-hole sums of a probe set against the extended plan's
+    (1e-8), execute's and the gradient's: no further off than the chain on complex GEMMs was with
+    these pupils. The tensor-core accumulator cuts every sum off; small products first keep that down."""
+    n, md, lams, states = 300, 201, np.linspace(500e-9, 600e-9, 5), 2
+    k = (np.arange(n) - n // 2) / n
+    u = np.random.default_rng(1).uniform(-1.0, 1.0, (6, 3))
+    opd = sum(5e-9 * a * np.cos(2 * np.pi * (3 * fx * k[None, :] + 3 * fy * k[:, None]) + 6 * a) for a, fx, fy in u)
+    disk = k[None, :] ** 2 + k[:, None] ** 2 <= 0.25
+    items, pupils = [], []
+    for lam in lams:
+        r = 550e-9 / lam
+        for a in range(states):
+            items.append(dict(m_occ=int(np.rint(90 * r)), du_occ=12.8 / 90 * r, spot_radius=5.0 * r, du_det=128.0 / md * r,
+                              dh_in=6.0 * r, dh_out=20.0 * r))
+            probe = 20e-9 * np.sinc(24 * k)[:, None] * (np.sinc(24 * k) * np.cos(26 * np.pi * k + a * np.pi / 4))[None, :]
+            pupils.append(disk * np.exp(2j * np.pi / lam * (opd + probe)))
+    x = torch.from_numpy(np.stack(pupils).astype(np.complex64)).cuda()
+    sums = {}
+    for p in (coro.MFT_EXT, prec):
+        plan = coro.LyotPlan(ctx, n=n, npix=float(n), lyot_frac=0.8, m_det=md, items=items, precision=p)
+        peak = plan.peak(x)
+        sums[p] = [plan.execute(x, peak=peak), plan.gradient(x, peak)[1]]
+        plan.close()
+    for got, ref in zip(sums[prec], sums[coro.MFT_EXT]):
+        err = np.sqrt(np.mean((got / ref - 1) ** 2))
+        print(f"prec {prec}: dark-hole sums off by {err:.3e}")
+        assert err < bar
