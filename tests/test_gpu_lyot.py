@@ -327,6 +327,11 @@ def test_broadband_batch_sampled_items(ctx, prec):
     plan.use_graph(False)
 
 
+def test_lyot_full_size_bf16_holds_three_planes(ctx):
+    """Between the dark-hole errors of two planes (1.04e-9) and of three (4.8e-10)."""
+    assert full_size_error(ctx, coro.MFT_3XBF16) < 8e-10
+
+
 @pytest.mark.parametrize("prec,bar", [(coro.MFT_3XTF32, 1.46e-5), (coro.MFT_3XBF16, 1.44e-5)])
 def test_darkhole_sums_are_as_close_as_with_complex_products(ctx, prec, bar):
     """Relative error (RMS over the items) of the dark-hole sums of a probe set against the extended plan's

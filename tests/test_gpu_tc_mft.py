@@ -83,3 +83,16 @@ def test_ext_mft_degenerate_inputs(ctx):
     err = rel_l2(y[0], propagation.mft(g[0].astype(np.complex64).astype(np.complex128), npix, m, du))
     print(f"EXT twelve-decade rows: rel L2 {err:.3e}")
     assert err < TOL[coro.MFT_EXT]
+
+
+@pytest.mark.parametrize("n,m,batch", [(64, 40, 2), (61, 500, 3), (300, 64, 1), (513, 129, 1), (1000, 301, 1)])
+def test_bf16_holds_three_planes(ctx, n, m, batch):
+    """3xBF16 keeps its third plane (24 bits): under the bar that two planes miss (test_split_formats.py)."""
+    from test_split_formats import BF16_BAR
+    f = inputs.random_field((batch, n, n), seed=n).astype(np.complex64)
+    du = np.linspace(0.2, 0.5, batch)
+    x = torch.from_numpy(f).cuda()
+    for d, ref in ((-1, propagation.mft), (+1, propagation.imft)):
+        y = coro.propagate_mft(ctx, x, 0.9 * n, d, m, du, coro.MFT_3XBF16).cpu().numpy()
+        for b in range(batch):
+            assert rel_l2(y[b], ref(f[b].astype(np.complex128), 0.9 * n, m, du[b])) < BF16_BAR
