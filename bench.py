@@ -835,7 +835,7 @@ def main():
         plan.set_pass_kernel(rv, cl)
     n_pass = plan.launch_count
     info = [plan.pass_info(i) for i in range(n_pass)]
-    flops = [plan.pass_flops(i) for i in range(n_pass)]
+    flops = [plan.pass_flops(i) * plan.pass_lines(i) / n for i in range(n_pass)]
     kernels = [plan.pass_kernel(i) for i in range(n_pass)]
     field = torch.empty((1, n, n), dtype=torch.complex64, device=device)
 
@@ -895,7 +895,7 @@ def main():
         return {"achieved": f_k / (t_k / 1e3) / 1e12, "peak": alu_peak, "unit": "TFLOP/s",
                 "frac": f_k / (t_k / 1e3) / 1e12 / alu_peak, "flops_per_launch": f_k / kinds[kind][2],
                 "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flops x {sm_max:.0f} MHz (derived)",
-                "flops": "5 N log2 N per line transform, 1 or 2 transforms per pass; elements not counted"}
+                "flops": "5 N log2 N per line that is transformed, 1 or 2 transforms per pass; elements not counted"}
     dom = max(kinds, key=lambda k: kinds[k][0])
     t_dom, b_dom, l_dom, k_dom = kinds[dom][:4]
     k_name = ", ".join(sorted(k_dom))

@@ -268,11 +268,16 @@ coro_status coro_plan_launch_count(coro_plan plan, int* out);
  * order for one on the alternating layout (coro_fresnel_plan_set_layout). */
 coro_status coro_fresnel_plan_execute_range(coro_plan plan, void* field, int first, int count);
 /* Describe pass i: *is_row (1 = row pass, 0 = column pass) and *bytes, the algorithmic HBM
- * traffic of the launch (field read unless generated, field write, OPD/amplitude maps read). */
+ * traffic of the launch (field read unless generated, field write, OPD/amplitude maps read; of the
+ * rows that the pass runs, where it leaves rows out). */
 coro_status coro_fresnel_plan_pass_info(coro_plan plan, int i, int* is_row, double* bytes);
-/* *flops: the pass's line transforms at the conventional 5 N log2 N real flops each (N lines
- * per item, one or two transforms per pass), elements and tables not counted. */
+/* *flops: the pass's line transforms over the whole field at the conventional 5 N log2 N real flops
+ * each (N lines per item, one or two transforms per pass), elements and tables not counted. */
 coro_status coro_fresnel_plan_pass_flops(coro_plan plan, int i, double* flops);
+/* *lines: the lines of each item that pass i transforms as the plan runs: n, or fewer in a row pass
+ * that leaves out the rows which masks make zero (coro_fresnel_plan_set_layout). The pass then does
+ * *lines / n of coro_fresnel_plan_pass_flops. Plain host query. */
+coro_status coro_fresnel_plan_pass_lines(coro_plan plan, int i, int* lines);
 /* Kernel that pass i launches, as chosen when the plan was built (the complex64 plan times
  * its candidates then unless the environment sets CORO_AUTOTUNE=0). *persistent:
  *   0  one block per group of lines;

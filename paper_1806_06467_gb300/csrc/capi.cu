@@ -1655,23 +1655,38 @@ extern "C" coro_status coro_fresnel_plan_pass_flops(coro_plan plan, int i, doubl
     return CORO_OK;
 }
 
+extern "C" coro_status coro_fresnel_plan_pass_lines(coro_plan plan, int i, int* lines) {
+    clear_error();
+    if (!plan || plan->kind() != 1 || !lines) { set_error("coro_fresnel_plan_pass_lines: bad argument"); return CORO_EINVAL; }
+    auto* p = static_cast<FresnelPlan*>(plan);
+    if (i < 0 || i >= (int)p->ops.size()) { set_error("coro_fresnel_plan_pass_lines: pass %d of %d", i, (int)p->ops.size()); return CORO_EINVAL; }
+    const Op& op = p->ops[i];
+    *lines = op.row && op.row_hi ? op.row_hi - op.row_lo : p->n;
+    return CORO_OK;
+}
+
 extern "C" coro_status coro_fresnel_plan_pass_info(coro_plan plan, int i, int* is_row, double* bytes) {
     clear_error();
     if (!plan || plan->kind() != 1 || !is_row || !bytes) { set_error("coro_fresnel_plan_pass_info: bad argument"); return CORO_EINVAL; }
     auto* p = static_cast<FresnelPlan*>(plan);
     if (i < 0 || i >= (int)p->ops.size()) { set_error("coro_fresnel_plan_pass_info: pass %d of %d", i, (int)p->ops.size()); return CORO_EINVAL; }
     const Op& op = p->ops[i];
-    const double field = (double)p->batch * p->n * p->n * (p->dtype == CORO_C64 ? 8.0 : 16.0);
-    const double plane = (double)p->n * p->n * 4.0;
-    double b = field;                                   // write
-    if (!op.row || !(op.row_flags & RF_INIT_ONE)) b += field;   // read
+    // what the launch moves: the rows (boxes of rows) that it runs, zeros of left-out rows where it writes them
+    const double n = p->n, row = (double)p->batch * n * (p->dtype == CORO_C64 ? 8.0 : 16.0);
+    const double box = col_box_rows(p->n), run = op.row_hi ? op.row_hi - op.row_lo : n;
+    double b = 0.0;
     if (op.row) {
+        if (!(op.row_flags & RF_INIT_ONE)) b += run * row;                 // read
+        b += (op.row_flags & RF_ZERO_REST ? n : run) * row;                // write
         for (int k = 0; k < op.elems.count; ++k) {
             const DevElem& e = op.elems.e[k];
             if (e.kind != DK_OPD_MAP) continue;
             const double maps = e.map_bstride ? (double)p->batch : 1.0;
-            b += plane * maps * (e.amp ? 2.0 : 1.0);
+            b += run * n * 4.0 * maps * (e.amp ? 2.0 : 1.0);
         }
+    } else {
+        b += (op.in_hi ? (op.in_hi - op.in_lo) * box : n) * row;
+        b += (op.out_hi ? (op.out_hi - op.out_lo) * box : n) * row;
     }
     *is_row = op.row ? 1 : 0;
     *bytes = b;

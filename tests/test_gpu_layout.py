@@ -290,3 +290,31 @@ def test_interleaved_row_pairs_match_natural_layout(ctx, n, batch):
         from oracle import optics
         ref = propagation.angular_spectrum(f[0] * optics.circular_aperture(n, dx, 0.3), dx, lam[0], z[0])
         assert np.linalg.norm(stored[0][0].cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,box", [(1024, 256), (2048, 256), (4096, 256), (1400, 200), (2800, 200), (4100, 410)])
+def test_pass_queries_count_the_rows_that_run(ctx, n, box, monkeypatch):
+    """Bytes and lines of the passes of a plan that leaves out rows behind its aperture and stop, and of
+    the same plan on every row."""
+    monkeypatch.setenv("CORO_AUTOTUNE", "0")
+    dx, r_ap, r_stop, batch = 1.0 / n, 0.1251, 0.0601, 2
+    m = torch.zeros((n, n), dtype=torch.float32, device="cuda")
+    els = [coro.element(coro.EL_OPD_MAP, plane=0, opd=m), coro.element(coro.EL_APERTURE, plane=0, radius=r_ap),
+           coro.element(coro.EL_OPD_MAP, plane=1, opd=m, amplitude=m), coro.element(coro.EL_CIRCLE, plane=2, radius=r_stop)]
+
+    def rows(r):                                         # a band of whole boxes around the middle
+        k = int(r * n)
+        return ((n // 2 + k + box) // box - (n // 2 - k) // box) * box
+
+    row = 8.0 * n * batch
+    for layout in (None, "0"):
+        monkeypatch.delenv("CORO_LAYOUT", raising=False) if layout is None else monkeypatch.setenv("CORO_LAYOUT", layout)
+        a, s = (rows(r_ap), rows(r_stop)) if layout is None else (n, n)
+        plan = coro.FresnelPlan(ctx, n=n, batch=batch, pixelscale=dx, wavelength=550e-9, distances=[1.5, 2.0], elements=els,
+                                init_uniform=True)
+        assert [plan.pass_lines(i) for i in range(plan.launch_count)] == [a, n, n, n, s]
+        want = [a * row + 4.0 * a * n,                   # field written, map read
+                (a + n) * row, 2 * n * row + 8.0 * n * n, (n + s) * row,
+                (s + n) * row]                           # the last pass writes zeros outside the stop's rows
+        assert [plan.pass_info(i)[1] for i in range(plan.launch_count)] == want
+        plan.close()
