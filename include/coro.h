@@ -275,7 +275,7 @@ coro_status coro_fresnel_plan_pass_info(coro_plan plan, int i, int* is_row, doub
  * each (N lines per item, one or two transforms per pass), elements and tables not counted. */
 coro_status coro_fresnel_plan_pass_flops(coro_plan plan, int i, double* flops);
 /* *lines: the lines of each item that pass i transforms as the plan runs: n, or fewer in a row pass
- * that leaves out the rows which masks make zero (coro_fresnel_plan_set_layout). The pass then does
+ * that leaves out the rows which masks make zero (see coro_fresnel_plan_set_layout). The pass does
  * *lines / n of coro_fresnel_plan_pass_flops. Plain host query. */
 coro_status coro_fresnel_plan_pass_lines(coro_plan plan, int i, int* lines);
 /* Kernel that pass i launches, as chosen when the plan was built (the complex64 plan times
@@ -319,20 +319,20 @@ coro_status coro_fresnel_plan_pass_radix(coro_plan plan, int i, int* radices, in
  * Every choice gives the same result up to FP32 rounding order (used to test each kernel). */
 coro_status coro_fresnel_plan_set_pass_kernel(coro_plan plan, int row_variant, int col_lines);
 /* (set_pass_kernel also returns the plan to the natural layout.)
- * Plane layout between passes (complex64 plans, n = 1024, 2048, 4096). Natural (0): every
- * pass transforms the field in place, column passes reading and writing strided column
- * pairs. Alternating (1): a column pass followed by a row pass writes its result transposed
- * ([b][x][y], contiguous rows) into a plane the plan owns (batch x n x n complex64, allocated
- * here, freed on return to 0 or with the plan), and the row pass reads it back column-wise
- * and writes the field's rows; each pass then has one strided side. Results agree up to FP32
- * rounding order. A plan starts on neither: at creation it takes the natural passes its tuner
- * picked, or (when faster, and without tuning) the packed-pair kernels with row pairs held
- * sample by sample interleaved between passes, in place, reported as layout 0; results are
- * bitwise those of the same kernels on the natural layout. There, and on the packed-pair engine
- * of n = 1400, 2800, 4100, rows that apertures and stops make zero are left out. The environment
- * sets CORO_LAYOUT=0 to keep natural rows throughout and every one of them, CORO_LAYOUT=1 for the alternating layout.
- * CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a
- * supported size. */
+ * Plane layout between passes. As created (0): a plan runs the natural passes its tuner picked, every
+ * pass transforming the field in place, column passes reading and writing strided column pairs; or, at
+ * n = 1024, 2048, 4096 in complex64, when faster and without tuning, the packed-pair kernels with row
+ * pairs held sample by sample interleaved between passes, in place, with results that are bitwise those
+ * of the same kernels on the natural layout. On interleaved row pairs, and on the packed-pair engine of
+ * n = 1400, 2800, 4100, rows that apertures and stops make zero are left out. Alternating (1; complex64,
+ * n = 1024, 2048, 4096): a column pass followed by a row pass writes its result transposed ([b][x][y],
+ * contiguous rows) into a plane the plan owns (batch x n x n complex64, allocated here, freed on return
+ * to 0 or with the plan), and the row pass reads it back column-wise and writes the field's rows; each
+ * pass then has one strided side. Results agree up to FP32 rounding order. Setting 0 returns to how
+ * the plan was created, or to natural passes on the kernels of coro_fresnel_plan_set_pass_kernel once
+ * that was called. The environment sets CORO_LAYOUT=0 to keep natural rows throughout and every one of
+ * them, CORO_LAYOUT=1 for the alternating layout.
+ * CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a supported size. */
 coro_status coro_fresnel_plan_set_layout(coro_plan plan, int transposed);
 /* Give dst the kernel choices and layout the tuner made for src (plans of the same dtype, n,
  * batch and pass sequence, e.g. a second buffer slot of one system): the two then run the

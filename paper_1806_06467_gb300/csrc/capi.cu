@@ -1114,6 +1114,7 @@ struct FresnelPlan : coro_plan_s {
     void* tbuf = nullptr;            // transposed plane of the alternating layout (owned)
     bool interleaved = false;        // ops run on interleaved row pairs (interleaved_ops)
     bool limited = false;            // ops leave rows out on the natural layout (mixed radix)
+    bool chosen = false;             // one of the two is how the plan was created: layout 0 returns to it
     RowLimits limits;
     DevBlocks db;
     std::vector<double> ps_final;
@@ -1156,8 +1157,17 @@ int transposed_ops(int dtype, int n, const std::vector<Op>& nat, std::vector<Op>
     return pairs;
 }
 
-// Switch a plan between the natural (0) and the alternating (1) layout. CORO_ENOTIMPL where
-// the plan has no column pass followed by a row pass at a size the pair kernels take.
+// Natural passes to how a plan runs without an alternating layout: on interleaved row pairs where there
+// are any, rows behind masks left out.
+void apply_choice(FresnelPlan* p) {
+    p->interleaved = interleaved_ops(p->dtype, p->n, p->ops_nat, &p->ops) > 0;
+    p->limited = !p->interleaved;
+    limit_rows(p->n, p->ops, p->limits);
+}
+
+// Switch a plan between layout 0 (how it was created; natural passes once their kernels were set) and
+// the alternating layout (1). CORO_ENOTIMPL where the plan has no column pass followed by a row pass at a
+// size the pair kernels take.
 coro_status set_layout(FresnelPlan* p, int transposed) {
     DeviceGuard g(p->device);
     std::vector<Op> t;
@@ -1180,6 +1190,7 @@ coro_status set_layout(FresnelPlan* p, int transposed) {
         }
     }
     p->interleaved = p->limited = false;
+    if (!transposed && p->chosen) apply_choice(p);
     p->graph.reset();                                   // a captured graph holds the old kernels
     return CORO_OK;
 }
@@ -1345,7 +1356,7 @@ void choose_layout(FresnelPlan* p) {
     if (!interleaved_ops(p->dtype, p->n, nat, &il)) {
         if (p->dtype != CORO_C64 || !(p->n & (p->n - 1))) return;
         limit_rows(p->n, p->ops, p->limits);
-        p->limited = true;
+        p->limited = p->chosen = true;
         return;
     }
     limit_rows(p->n, il, p->limits);
@@ -1363,7 +1374,7 @@ void choose_layout(FresnelPlan* p) {
     }
     p->ops_nat = nat;
     p->ops = il;
-    p->interleaved = true;
+    p->interleaved = p->chosen = true;
 }
 
 coro_status finish_plan(coro_ctx ctx, std::unique_ptr<FresnelPlan>& plan, coro_plan* out, const char* who) {
@@ -1742,6 +1753,7 @@ extern "C" coro_status coro_fresnel_plan_set_pass_kernel(coro_plan plan, int row
         if (op.row) op.variant = row_variant;
         else op.lines = col_lines;
     }
+    p->chosen = false;
     return set_layout(p, 0);                            // every pass in place with these kernels
 }
 
@@ -1763,14 +1775,9 @@ extern "C" coro_status coro_fresnel_plan_copy_tuning(coro_plan dst, coro_plan sr
         d->ops_nat[i].variant = s->ops_nat[i].variant;
         d->ops_nat[i].lines = s->ops_nat[i].lines;
     }
-    d->ops = d->ops_nat;
+    d->chosen = s->chosen;
     coro_status st = set_layout(d, 0);
     if (st == CORO_OK && s->tbuf) st = set_layout(d, 1);
-    if (st == CORO_OK && (s->interleaved || s->limited)) {
-        d->limited = s->limited;
-        d->interleaved = interleaved_ops(d->dtype, d->n, d->ops_nat, &d->ops) > 0;
-        limit_rows(d->n, d->ops, d->limits);
-    }
     return st;
 }
 

@@ -318,3 +318,34 @@ def test_pass_queries_count_the_rows_that_run(ctx, n, box, monkeypatch):
                 (s + n) * row]                           # the last pass writes zeros outside the stop's rows
         assert [plan.pass_info(i)[1] for i in range(plan.launch_count)] == want
         plan.close()
+
+
+@pytest.mark.parametrize("n", [1024, 4096])
+def test_layout_that_was_queried_brings_the_plan_back(ctx, n, monkeypatch):
+    """layout -> alternating -> the queried layout: the passes, left-out rows and bits the plan was
+    created with; a kernel set by hand stays what layout 0 returns to, and a copy follows its source."""
+    monkeypatch.setenv("CORO_AUTOTUNE", "0")
+    monkeypatch.delenv("CORO_LAYOUT", raising=False)
+    w = inputs.RelayWorkload(n=n, npix=n // 4, seed=12)
+    maps_t = [torch.from_numpy(m.astype(np.float32)).cuda() for m in w.psd_maps()]
+    plan, other = relay_plan(ctx, w, maps_t), relay_plan(ctx, w, maps_t)
+
+    def state(p):
+        x = torch.full((1, n, n), float("nan"), dtype=torch.complex64, device="cuda")
+        p.execute(x)
+        return names(p), [p.pass_lines(i) for i in range(p.launch_count)], [p.pass_info(i) for i in range(p.launch_count)], x
+
+    a, was = state(plan), plan.layout
+    assert a[1][0] < n and not was
+    plan.set_layout(True)
+    assert plan.layout and state(plan)[1] == [n] * plan.launch_count
+    other.copy_tuning(plan)
+    assert other.layout
+    for p in (plan, other):
+        p.set_layout(was)
+        b = state(p)
+        assert a[:3] == b[:3] and torch.equal(a[3], b[3])
+    plan.set_pass_kernel(1, 0)
+    plan.set_layout(True)
+    plan.set_layout(False)
+    assert state(plan)[1] == [n] * plan.launch_count and not any("_pair" in k for k in names(plan) if k.startswith("row"))
