@@ -228,6 +228,10 @@ ft_gemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
                     if (++s == stages) { s = 0; ph ^= 1; }
                 }
             }
+            // no copy is in flight when the block ends, whatever wait expired: the last load of each stage
+            // (a stage never loaded passes, its barrier being in its first phase)
+#pragma unroll 1
+            for (int x = 0; x < stages; ++x) tc::mbar_wait(&full[x], x < s ? ph : ph ^ 1, a.err, 25);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -305,6 +309,8 @@ ft_gemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
                     }
                 }
             }
+            // nor is an MMA, when the tensor memory is given back
+            tc::mbar_wait(&empty[(s ? s : stages) - 1], s ? ph : ph ^ 1, a.err, 26);
         }
     } else {
         const int q = warp & 3;                      // TMEM lane quarter this warp may read

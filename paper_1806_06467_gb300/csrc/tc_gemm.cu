@@ -104,7 +104,8 @@ tc_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ 
 
     if (warp == 0) {
         if (lane == 0) {
-            for (int k = 0; k < kblocks; ++k) {
+            int k = 0;
+            for (; k < kblocks; ++k) {
                 const int s = k % STAGES;
                 const uint32_t ph = (k / STAGES) & 1;
                 if (!tc::mbar_wait(&empty[s], ph ^ 1, a.err, 1)) break;
@@ -113,6 +114,8 @@ tc_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ 
                 tc::tma_load_4d(st, &mx, &full[s], (kb0 + k) * KE, m0, 0, it.x_idx);
                 tc::tma_load_4d(st + OPER_BYTES, &mw, &full[s], (kb0 + k) * KE, n0, 0, it.w_idx);
             }
+            // no copy is in flight when the block ends, whatever wait expired
+            for (int x = k > STAGES ? k - STAGES : 0; x < k; ++x) tc::mbar_wait(&full[x % STAGES], (x / STAGES) & 1, a.err, 5);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -122,7 +125,8 @@ tc_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ 
             constexpr uint32_t ID_POS = tc::idesc<BF16>(BM, BN, false);
             constexpr uint32_t ID_NEG = tc::idesc<BF16>(BM, BN, true);
             bool ok = true;
-            for (int k = 0; k < kblocks && ok; ++k) {
+            int k = 0;
+            for (; k < kblocks; ++k) {
                 const int s = k % STAGES;
                 const uint32_t ph = (k / STAGES) & 1;
                 const int c = k / kChunk, buf = c & 1, kc = k % kChunk;
@@ -154,6 +158,8 @@ tc_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ 
                 tc::umma_commit(&empty[s]);             // frees the stage once these MMAs retire
                 if (kc == kChunk - 1 || k == kblocks - 1) tc::umma_commit(&tfull[buf]);
             }
+            // nor is an MMA, when the tensor memory is given back
+            if (k) tc::mbar_wait(&empty[(k - 1) % STAGES], ((k - 1) / STAGES) & 1, a.err, 6);
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..9)

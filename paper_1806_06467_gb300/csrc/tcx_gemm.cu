@@ -164,6 +164,9 @@ tcx_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__
                     tc::tma_load_4d(st + X_BYTES, &mw, &full[s], kx, tl.n0, 0, it.w_idx);
                 }
             }
+            // no copy is in flight when the block ends, whatever wait expired
+            for (long long x = kk > STAGES ? kk - STAGES : 0; x < kk; ++x)
+                tc::mbar_wait(&full[x % STAGES], (uint32_t)(x / STAGES) & 1, a.err, 15);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -215,6 +218,8 @@ tcx_cgemm_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__
             }
             gg += tl.ngroups;
             }
+            // nor is an MMA, when the tensor memory is given back
+            if (kk) tc::mbar_wait(&empty[(kk - 1) % STAGES], (uint32_t)((kk - 1) / STAGES) & 1, a.err, 16);
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..17)
