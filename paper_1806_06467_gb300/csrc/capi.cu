@@ -1870,11 +1870,11 @@ __device__ __forceinline__ float intensity_of(float2 v, double s, float sh, floa
     const float p = v.x * v.x, q = v.y * v.y, h = p + q;
     if (v.x == 0.f && v.y == 0.f) return 0.f;            // outside a stop; s is finite
     const float r = h * sh;
+    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f)) return intensity_fp64(v, s);
     const float ep = fmaf(v.x, v.x, -p), eq = fmaf(v.y, v.y, -q), bb = h - p;
     const float l = ((p - (h - bb)) + (q - bb)) + (ep + eq);
     const float t = fmaf(h, sh, -r) + (h * sl + l * sh), up = r + fmaf(r, 0x1p-43f, t);
-    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f && up == r + fmaf(r, -0x1p-43f, t))) return intensity_fp64(v, s);
-    return up;
+    return up == r + fmaf(r, -0x1p-43f, t) ? up : intensity_fp64(v, s);
 }
 
 // grid.y: items. Two samples per thread and step where they sit on a 16-byte boundary.
