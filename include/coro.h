@@ -319,19 +319,20 @@ coro_status coro_fresnel_plan_pass_radix(coro_plan plan, int i, int* radices, in
  * Every choice gives the same result up to FP32 rounding order (used to test each kernel). */
 coro_status coro_fresnel_plan_set_pass_kernel(coro_plan plan, int row_variant, int col_lines);
 /* (set_pass_kernel also returns the plan to the natural layout.)
- * Plane layout between passes. As created (0): a plan runs the natural passes its tuner picked, every
- * pass transforming the field in place, column passes reading and writing strided column pairs; or, at
- * n = 1024, 2048, 4096 in complex64, when faster and without tuning, the packed-pair kernels with row
- * pairs held sample by sample interleaved between passes, in place, with results that are bitwise those
- * of the same kernels on the natural layout. On interleaved row pairs, and on the packed-pair engine of
- * n = 1400, 2800, 4100, rows that apertures and stops make zero are left out. Alternating (1; complex64,
- * n = 1024, 2048, 4096): a column pass followed by a row pass writes its result transposed ([b][x][y],
- * contiguous rows) into a plane the plan owns (batch x n x n complex64, allocated here, freed on return
- * to 0 or with the plan), and the row pass reads it back column-wise and writes the field's rows; each
- * pass then has one strided side. Results agree up to FP32 rounding order. Setting 0 returns to how
- * the plan was created, or to natural passes on the kernels of coro_fresnel_plan_set_pass_kernel once
- * that was called. The environment sets CORO_LAYOUT=0 to keep natural rows throughout and every one of
- * them, CORO_LAYOUT=1 for the alternating layout.
+ * Plane layout between passes. As created (0): a plan runs the natural passes its tuner picked,
+ * every pass transforming the field in place, column passes reading and writing strided column
+ * pairs; or, at n = 1024, 2048, 4096 in complex64, when faster and without tuning, the packed-pair
+ * kernels with row pairs held sample by sample interleaved between passes, in place, with results
+ * that are bitwise those of the same kernels on the natural layout. On interleaved row pairs, and
+ * on the packed-pair engine of n = 1400, 2800, 4100, rows that apertures and stops make zero are
+ * left out. Alternating (1; complex64, n = 1024, 2048, 4096): a column pass followed by a row pass
+ * writes its result transposed ([b][x][y], contiguous rows) into a plane the plan owns (batch x
+ * n x n complex64, allocated here, freed on return to 0 or with the plan), and the row pass reads
+ * it back column-wise and writes the field's rows; each pass then has one strided side. Results
+ * agree up to FP32 rounding order. Setting 0 returns to how the plan was created, or to natural
+ * passes on the kernels of coro_fresnel_plan_set_pass_kernel once that was called. The environment
+ * sets CORO_LAYOUT=0 to keep natural rows throughout and every one of them, CORO_LAYOUT=1 for the
+ * alternating layout at creation (0 is then the natural one).
  * CORO_ENOTIMPL: the plan has no column pass followed by a row pass at a supported size. */
 coro_status coro_fresnel_plan_set_layout(coro_plan plan, int transposed);
 /* Give dst the kernel choices and layout the tuner made for src (plans of the same dtype, n,
@@ -374,7 +375,7 @@ coro_status coro_plan_destroy(coro_plan plan);
  * runs in rounds, so that they stay within 2 GiB where one item's are smaller than that.
  * ------------------------------------------------------------------------------------------ */
 typedef enum {
-    CORO_MFT_FP32 = 0,    /* FP32 CUDA-core complex GEMM                                     */
+    CORO_MFT_FP32 = 0,    /* FP32 CUDA cores, on even / odd halves with real bases           */
     CORO_MFT_3XTF32 = 1,  /* split TF32 tensor-core GEMM (hi*hi + hi*lo + lo*hi), FP32 acc   */
     CORO_MFT_3XBF16 = 2,  /* split BF16 tensor-core GEMM, FP32 accumulate (three planes, six */
                           /* products; two planes, three products in complex GEMMs)          */
@@ -417,8 +418,9 @@ coro_status coro_dm_correlate(coro_ctx ctx, const float* w, int batch, int n, do
  * plane with real bases (a quarter of the complex products; planes trimmed to the spot and the
  * stop); spot, Babinet subtraction and Lyot stop are fused into GEMM epilogues, intensity and
  * dark-hole sum into the kernel that leaves the halves. Where a mask reaches the unpaired sample of
- * an even axis (index 0, coordinate -n/2), complex GEMMs with the intensity fused run instead. Items may have different
- * occulter sizes m_occ (uneven per-wavelength sampling); n, npix, lyot_frac, m_det are shared.
+ * an even axis (index 0, coordinate -n/2), complex GEMMs with the intensity fused run instead, for
+ * the whole batch. Items may have different occulter sizes m_occ (uneven per-wavelength sampling);
+ * n, npix, lyot_frac, m_det are shared.
  * The plan owns its work buffers (bases, split operands) for its lifetime.
  * ------------------------------------------------------------------------------------------ */
 typedef struct {
@@ -448,8 +450,8 @@ typedef struct {
 coro_status coro_lyot_plan_create(coro_ctx ctx, const coro_lyot_desc* desc, coro_plan* out);
 /* pupil: device complex64 [batch][n][n] (E_A; complex128 for CORO_MFT_FP64). peak: host [batch]
  * normalisation (NULL = 1). intensity: device float [batch][m_det][m_det] or NULL. field: device
- * complex64 (complex128 for CORO_MFT_FP64) [batch][m_det][m_det] (unnormalised E_det) or NULL. dh: host [batch] dark-hole sums or NULL
- * (when given, the stream is synchronised). */
+ * complex64 (complex128 for CORO_MFT_FP64) [batch][m_det][m_det] (unnormalised E_det) or NULL. dh:
+ * host [batch] dark-hole sums or NULL (when given, the stream is synchronised). */
 coro_status coro_lyot_plan_execute(coro_plan plan, const void* pupil, const double* peak, float* intensity,
                                    void* field, double* dh);
 /* `times` executes back to back (one graph when graphs are on), without the host copy of dh;
@@ -461,8 +463,8 @@ coro_status coro_lyot_plan_execute_n(coro_plan plan, const void* pupil, const do
 coro_status coro_lyot_plan_peak(coro_plan plan, const void* pupil, double* peak_out);
 /* Run stages [first, first + count) only (for per-launch timing): 0 split of the pupil, 1-4 the
  * GEMMs pupil->occulter (two), occulter->Lyot with Babinet (two), 5 the detector MFT with its
- * intensity (two GEMMs and, on halves, the kernel that leaves them; a stream memset of the
- * dark-hole sums comes first).
+ * intensity (two GEMMs; on halves also the kernel that leaves them and writes the dark-hole sums,
+ * in complex GEMMs a stream memset of those sums first).
  * Running 0-5 in order equals coro_lyot_plan_execute without the host copy of dh. */
 coro_status coro_lyot_plan_execute_range(coro_plan plan, const void* pupil, const double* peak, float* intensity,
                                          void* field, int first, int count);

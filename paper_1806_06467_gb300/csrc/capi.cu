@@ -1867,13 +1867,13 @@ namespace {
 __device__ __noinline__ float intensity_fp64(float2 v, double s) { return (float)(((double)v.x * v.x + (double)v.y * v.y) * s); }
 
 __device__ __forceinline__ float intensity_of(float2 v, double s, float sh, float sl) {
-    const float p = v.x * v.x, q = v.y * v.y, h = p + q;
-    if (v.x == 0.f && v.y == 0.f) return 0.f;            // outside a stop; s is finite
-    const float r = h * sh;
-    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f)) return intensity_fp64(v, s);
-    const float ep = fmaf(v.x, v.x, -p), eq = fmaf(v.y, v.y, -q), bb = h - p;
-    const float l = ((p - (h - bb)) + (q - bb)) + (ep + eq);
-    const float t = fmaf(h, sh, -r) + (h * sl + l * sh), up = r + fmaf(r, 0x1p-43f, t);
+    const float p = v.x * v.x, q = v.y * v.y, h = p + q, r = h * sh;
+    if (!(h > 1e-30f && h < 1e30f && r > 1e-30f && r < 1e30f)) {
+        if (v.x == 0.f && v.y == 0.f) return 0.f;        // outside a stop; s is finite
+        return intensity_fp64(v, s);
+    }
+    const float l = ((fmaxf(p, q) - h) + fminf(p, q)) + (fmaf(v.x, v.x, -p) + fmaf(v.y, v.y, -q));
+    const float t = fmaf(h, sh, -r) + fmaf(h, sl, l * sh), up = r + fmaf(r, 0x1p-43f, t);
     return up == r + fmaf(r, -0x1p-43f, t) ? up : intensity_fp64(v, s);
 }
 

@@ -38,7 +38,7 @@ enum FoldEpi : int {
 // One contraction of `items` planes (grid z = item x parity).
 //   X [item][2][K][M]  complex, M = 2 Hm: (parity, index) of the other axis; item stride sX
 //   W [item][2][K][ldw] real, zero-filled beyond N up to ldw (a multiple of 32); item stride sW
-//   Y [item][M][2][N]  complex; item stride sY; split s of K writes at Y + s * sSplit
+//   Y [item][M][2][N]  complex; item stride sY (K splits: partial planes in `part`, then summed)
 // base (FOLD_BABINET): class plane [2][base_h][2][base_h] read at (parity m, index m, p, n).
 template <typename C>
 struct FoldGemm {

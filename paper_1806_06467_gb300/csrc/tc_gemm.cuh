@@ -123,7 +123,8 @@ cudaError_t tc_launch(bool bf16, int epi, const CUtensorMap& mx, const CUtensorM
 cudaError_t tc_split(bool bf16, const float2* src, long long src_bstride, int src_ld, const TcOperand& dst,
                      cudaStream_t stream, const int* keep_r2 = nullptr);
 // W[r][k] = exp(sign 2 pi i (r - rows/2)(k - cols/2) c) straight into planar split form: one basis
-// (index `item` of dst), rows_valid x cols_valid centred on their own halves; everything else in that item's planes is left untouched
+// (index `item` of dst), rows_valid x cols_valid centred on their own halves; everything else in
+// that item's planes is left untouched
 cudaError_t tc_basis_one(bool bf16, double c, int sign, const TcOperand& dst, int item, int rows_valid,
                          int cols_valid, cudaStream_t stream);
 // planar split operand -> complex64 (hi + lo), dst[b * dst_bstride + r * dst_ld + k]
